@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256, L * C <= 4 ? 4 : (L * C <= 8 ? 3 : 2)) k_
   __shared__ uint32_t tmem_slot;
   __shared__ volatile uint32_t abort_flag;
   __shared__ volatile uint32_t stop_flag[2];  // the consumer's decision for tile j, in slot j & 1
-  const uint32_t tid = threadIdx.x, row = tid & 127, wg = tid >> 7;
+  const uint32_t tid = threadIdx.x, row = tid & 127, warp = uniform(tid >> 5), wg = warp >> 2;
   const uint32_t lanes = ((row >> 5) * 32) << 16;  // this warp's TMEM lane quadrant
   constexpr int NF = L * C + 4 * kGenMaxPe;  // feature values this input layout can have
   constexpr int NP = (NF + 15) / 16 * 16;
@@ -155,9 +155,9 @@ __global__ void __launch_bounds__(256, L * C <= 4 ? 4 : (L * C <= 8 ? 3 : 2)) k_
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tAcc = tmem_slot;             // H fp32 columns
-  const uint32_t tAH = tmem_slot + H;          // hidden A operand, H / 2 columns
-  const uint32_t tA1 = tmem_slot + H + H / 2;  // ring stages, K1 / 2 columns each
+  const uint32_t tAcc = uniform(tmem_slot);  // H fp32 columns
+  const uint32_t tAH = tAcc + H;             // hidden A operand, H / 2 columns
+  const uint32_t tA1 = tAcc + H + H / 2;     // ring stages, K1 / 2 columns each
   const uint32_t T = __ldg(B.meta);
   const bool copied = rows_copied(B, D);
   const uint32_t grid = gridDim.x;
@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(256, L * C <= 4 ? 4 : (L * C <= 8 ? 3 : 2)) k_
     // ------------------------------------------------------------- consumer
     uint32_t cur = 0xFFFFFFFFu, mph = 0, wph = 0;
     const uint32_t sW = saddr(smem);
+    const bool mma_warp = (warp & 3) == 0;  // its elected lane issues the MMAs
     TileWalk cwalk;
     const uint32_t id_h = instr_desc<BF16>(H), id_o = instr_desc<BF16>(16);
     const uint32_t act = G.activation == 1 && G.slope >= 0.0f && G.slope <= 1.0f ? 2u : G.activation;
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(256, L * C <= 4 ? 4 : (L * C <= 8 ? 3 : 2)) k_
         wph ^= 1;
         cur = dec;
       }
-      if (row == 0) {
+      if (mma_warp && elect_one()) {
         fence_after();
         const uint64_t d1 = smem_desc(sW, K1);
         for (uint32_t kc = 0; kc < K1 / 16; ++kc)
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(256, L * C <= 4 ? 4 : (L * C <= 8 ? 3 : 2)) k_
         tmem_wait_st();
         fence_before();
         wg_bar(1);
-        if (row == 0) {
+        if (mma_warp && elect_one()) {
           fence_after();
           const bool last = l + 1 == NL;
           const uint64_t dw = smem_desc(sW + gen_w_off(G, l + 1), H);

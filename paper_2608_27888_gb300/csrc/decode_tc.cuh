@@ -348,7 +348,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
   using M = TmSmem<H, NC, SC>;
   using TC = TmCols<H, NC, SC>;
   extern __shared__ __align__(128) uint8_t smem[];
-  const int role = threadIdx.x >> 7, row = threadIdx.x & 127, warp = threadIdx.x >> 5;
+  const int warp = (int)uniform(threadIdx.x >> 5), role = warp >> 2, row = threadIdx.x & 127;
   const int lane = threadIdx.x & 31;
   const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;  // this warp's TMEM lane quadrant
   const uint32_t sbase = saddr(smem);
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = uniform(*tmem_slot);
   const uint32_t one = BF16 ? 0x3F80u : 0x3C00u;  // 1.0 in the low half, 0 in the high half
   if (warp < 4) {  // the shared bias operand: K column 0 is 1, the rest 0
     const uint32_t z[8] = {one, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
@@ -556,6 +556,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
     // ------------------------------------------------------------ consumer
     const int c = role - NP;
     const int wgid = role;  // named barrier id role + 1
+    const bool mma_warp = (warp & 3) == 0;  // its elected lane issues the MMAs (no issuer warps)
     const bool poller = (row >> 5) == (c & 3);  // one waiting warp per consumer, spread over the sub-partitions
     const uint32_t tD = tmem_base + TC::acc(c);  // accumulator
     const uint32_t tH = tmem_base + TC::hid(c);  // hidden A operand
@@ -610,7 +611,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
           out_pending = false;
           wg_bar(wgid);
         }
-        if (row == 0) {
+        if (mma_warp && elect_one()) {
           fence_after();
           bulk_g2s(sW1, W.tc + (size_t)dec * W.tc_stride, L::WIMG, wbar);
         }
@@ -627,7 +628,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
       stop = stop_flag[2 * c + (jc & 1)] != 0;
       oi = reinterpret_cast<const uint32_t *>(smem + M::oidx)[(s * 2 + (n & 1)) * 128 + row];
       good = oi != 0xFFFFFFFFu;
-      if (row == 0) {
+      if (mma_warp && elect_one()) {
         fence_after();
         if (dec < D) {
           const uint32_t tA = tmem_base + TC::a1(s);
@@ -773,7 +774,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
             hidden();
             fence_before();
             wg_bar(wgid);
-            if (row == 0) {
+            if (mma_warp && elect_one()) {
               fence_after();
               if (layer == 0) {
 #pragma unroll
@@ -827,7 +828,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
     // prepares the next tile while the epilogue converts layer 2's result; B
     // issues the output layer's bias and first K steps once Y arrives and the
     // rest once Z arrives.  Every wait is bounded.
-    const int iw = (int)((threadIdx.x - (NP + NC) * 128) >> 5);
+    const int iw = warp - (NP + NC) * 4;
     const int c = iw >> 1;
     const bool issuer_a = (iw & 1) == 0;
     const uint32_t tD = tmem_base + TC::acc(c), tH = tmem_base + TC::hid(c), tOnes = tmem_base + TC::ONES;
@@ -891,6 +892,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
           stop_flag[2 * c + (jc & 1)] = stop;
         }
         if (swap) cur = dec;
+        __syncwarp();  // lane 0 waited for the weights, the elected lane issues
         stop = __shfl_sync(0xFFFFFFFFu, stop, 0);
         named_arrive(bT, kIssTN);
         return stop;
@@ -902,7 +904,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
         if (stop) break;
         const uint32_t tdec = dec;
         if (tdec < D) {
-          if (lane == 0) {
+          if (elect_one()) {
             fence_after();
             umma_ta(tD, tmem_base + TC::a1(s), dW1, id_hidden, 0);
             umma_ta(tD, tOnes, dW1 + 16, id_hidden, 1);  // + bias
@@ -916,7 +918,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
         __syncwarp();
         named_sync(bX, kIssXN);  // layer 1's result converted (or the bad tile taken over)
         if (tdec < D) {
-          if (lane == 0) {
+          if (elect_one()) {
             fence_after();
 #pragma unroll
             for (uint32_t kq = 0; kq < H / 16; ++kq) umma_ta(tD, tH + 8 * kq, dW2 + 16 * kq, id_hidden, kq);
@@ -940,7 +942,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
         if (stop_flag[2 * c + (jc & 1)]) break;
         if (dec >= D) continue;
         named_sync(bY, kIssYN);
-        if (lane == 0) {  // the bias, then the K steps of the converted half
+        if (elect_one()) {  // the bias, then the K steps of the converted half
           fence_after();
           umma_ta(tO, tOnes, dW3 + 16 * (H / 16), id_out, 0);
 #pragma unroll
@@ -949,7 +951,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
         issued = true;
         __syncwarp();
         named_sync(bZ, kIssZN);
-        if (lane == 0) {
+        if (elect_one()) {
           fence_after();
 #pragma unroll
           for (uint32_t kq = H / 32; kq < H / 16; ++kq) umma_ta(tO, tH + 8 * kq, dW3 + 16 * kq, id_out, 1);
@@ -958,7 +960,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
         __syncwarp();
       }
     }
-    if (lane == 0 && issued) {  // no MMA of this issuer is in flight when tensor memory is released
+    if (issued && elect_one()) {  // no MMA of this issuer is in flight when tensor memory is released
       umma_commit(fbar);
       wait(fbar, 0);
     }

@@ -51,6 +51,22 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 
+// One lane of the (fully converged) warp, the same lane every time.  MMAs are
+// issued under `if (elect_one())` inside warp-uniform control flow, with
+// operands that derive from uniform() values: tcgen05.mma takes its operands
+// from uniform registers, and the compiler then keeps them there.  Under
+// `if (threadIdx == 0)` it moves every operand across for each MMA: on GB300 one
+// thread issued four N = 64 MMAs and their commit in 305 cycles that way and in
+// 44 this way (completion 451 -> 225 cycles; N = 16: 453 -> 131; nine N = 128
+// MMAs are bound by the tensor pipe, 64 cycles each, either way).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xFFFFFFFF;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0;
+}
+// A value that is the same in every lane, in a form the compiler knows is.
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xFFFFFFFFu, x, 0); }
+
 __device__ __forceinline__ void fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
 }
