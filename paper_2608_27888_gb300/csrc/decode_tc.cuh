@@ -279,9 +279,29 @@ struct TmSmem {
   // full, empty, mma, weights, output; with issuer warps each issuer's final commit
   static constexpr int nbars = 2 * S + 3 * NC + (issuer_warp<H>() ? 2 * NC : 0);
   static constexpr size_t misc = bars + (size_t)nbars * 8;
-  static constexpr size_t tiles = misc + 64;
-  static constexpr size_t grids = tiles + 2 * kSmemTileTable * 4;
-  static constexpr size_t total = grids + kSmemGrids * sizeof(GridDesc);
+  static constexpr size_t tables = misc + 64;  // TmTables, sized by the launch
+};
+
+// What follows the fixed plan, at the size the launch needs and no more (what
+// is left of the SM's array is the L1 that holds the gathers): the grid table
+// and the tile table, if they fit their limits, and each consumer warp's row
+// buffer, if its rows are not written with one vector store each.
+struct TmTables {
+  uint32_t grids, tiles, rows, total;  // byte offsets in shared memory; total = all of it
+  uint32_t vector_rows;                // 1: a row is one vector store
+  uint32_t div_c;                      // k / C = k * div_c >> 16 for k < 512 (write_rows)
+  // rows of the buffer are padded to an odd number of words: no bank conflicts
+  static __host__ __device__ __forceinline__ uint32_t row_words(uint32_t C) { return C | 1u; }
+  static TmTables plan(size_t fixed, uint32_t ngrids, uint32_t D, uint32_t C, bool vector_rows, uint32_t row_warps) {
+    TmTables t;
+    t.grids = (uint32_t)((fixed + 15) / 16 * 16);
+    t.tiles = t.grids + (ngrids <= kSmemGrids ? ngrids : 0u) * (uint32_t)sizeof(GridDesc);
+    t.rows = t.tiles + (D + 2 <= kSmemTileTable ? 2 * (D + 2) : 0u) * 4;
+    t.vector_rows = vector_rows;
+    t.div_c = (65536 + C - 1) / C;
+    t.total = t.rows + (vector_rows ? 0u : row_warps) * 32 * row_words(C) * 4;
+    return t;
+  }
 };
 
 // Tensor-memory plan (columns).  The NC fp32 accumulators (H columns each)
@@ -309,6 +329,57 @@ struct TmCols {
   static __device__ __forceinline__ uint32_t a1(uint32_t s) { return STG + 8 * s; }
   static __device__ __forceinline__ uint32_t out(uint32_t c) { return OUT + 16 * c; }
 };
+
+__device__ __forceinline__ void put_elem(float *p, float y) { *p = y; }
+__device__ __forceinline__ void put_elem(__half *p, float y) { *p = __float2half_rn(y); }
+
+// A warp's 32 output rows of C elements, from its row buffer (row r of the
+// warp at r * TmTables::row_words(C)) to out: element k = lane + 32 i of the
+// 32 x C block in store i, so that a store covers consecutive elements of a few
+// rows.  Straight-line code without a carried row counter: the epilogue warps'
+// latency is on the decode's critical path.
+template <typename E>
+__device__ __forceinline__ void write_rows(E *out, const float *rowbuf, uint32_t C, uint32_t oi, bool good, int lane,
+                                           uint32_t div_c) {
+  const uint32_t oi0 = __shfl_sync(0xFFFFFFFFu, oi, 0);
+  const bool side_by_side = __all_sync(0xFFFFFFFFu, good && oi == oi0 + (uint32_t)lane);
+  if (side_by_side && (C & 1)) {  // the block is 32 C consecutive elements on both sides
+    E *p = out + (size_t)oi0 * C + lane;
+    const float *b = rowbuf + lane;
+#pragma unroll
+    for (uint32_t g = 0; g < 16; g += 3) {
+      if (g >= C) break;
+      float v[3];
+#pragma unroll
+      for (uint32_t j = 0; j < 3; ++j)
+        if (g + j < C) v[j] = b[32 * (g + j)];
+#pragma unroll
+      for (uint32_t j = 0; j < 3; ++j)
+        if (g + j < C) put_elem(p + 32 * (g + j), v[j]);
+    }
+    return;
+  }
+  const uint32_t row = good ? oi : 0xFFFFFFFFu, even = 1u - (C & 1u);
+#pragma unroll
+  for (uint32_t g = 0; g < 16; g += 3) {
+    if (g >= C) break;
+    float v[3];
+    uint32_t ro[3], ch[3];
+#pragma unroll
+    for (uint32_t j = 0; j < 3; ++j) {
+      const uint32_t k = (uint32_t)lane + 32 * (g + j), r = k * div_c >> 16;
+      ch[j] = k - r * C;
+      ro[j] = __shfl_sync(0xFFFFFFFFu, row, r & 31u);
+      if (g + j < C)
+        v[j] = rowbuf[k + even * r];
+      else
+        ro[j] = 0xFFFFFFFFu;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < 3; ++j)
+      if (ro[j] != 0xFFFFFFFFu) put_elem(out + (size_t)ro[j] * C + ch[j], v[j]);
+  }
+}
 
 // Warp-specialised gather-decode with tensor-memory operands.
 //   Consumer warpgroups (the last NC) each decode the CTA's local tiles
@@ -339,7 +410,7 @@ struct TmCols {
 template <int H, bool BF16, bool TRI, bool WRAP, int CP, int NP, int NC, int SC, bool DBG>
 __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 : 0), 1)
     k_decode_tm(Assets A, WeightImages W, Buckets B, void *out, unsigned long long *err,
-                unsigned int *status, int vec_out, ntc_debug_row *dbg) {
+                unsigned int *status, TmTables tb, ntc_debug_row *dbg) {
   static_assert(NP % NC == 0 && SC % (NP / NC) == 0, "each ring stage needs one producer");
   constexpr int R = NP / NC;  // producers per consumer
   constexpr bool ISS = issuer_warp<H>();
@@ -368,7 +439,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
   const GridDesc *grids = A.pgrids;  // grid bases in the row-pair copy
   const uint32_t ngrids = A.num_sets * kLevels * A.num_mips;
   if (ngrids <= kSmemGrids) {
-    GridDesc *s_grids = reinterpret_cast<GridDesc *>(smem + M::grids);
+    GridDesc *s_grids = reinterpret_cast<GridDesc *>(smem + tb.grids);
     for (uint32_t i = threadIdx.x; i < ngrids; i += blockDim.x) s_grids[i] = A.pgrids[i];
     grids = s_grids;
   }
@@ -403,8 +474,8 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
   pdl_wait();
   const uint32_t *seg = B.meta + 1, *tst = B.meta + 1 + (D + 2);
   if (!B.identity_n && D + 2 <= kSmemTileTable) {
-    uint32_t *s_seg = reinterpret_cast<uint32_t *>(smem + M::tiles);
-    uint32_t *s_tst = s_seg + kSmemTileTable;
+    uint32_t *s_seg = reinterpret_cast<uint32_t *>(smem + tb.tiles);
+    uint32_t *s_tst = s_seg + D + 2;
     for (uint32_t i = threadIdx.x; i < D + 2; i += blockDim.x) {
       s_seg[i] = __ldg(seg + i);
       s_tst[i] = __ldg(tst + i);
@@ -641,22 +712,34 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
         }
       }
     };
-    // the sigmoid epilogue of one tile: its output accumulator(s) -> out[eoi]
+    // The sigmoid epilogue of one tile: its output accumulator -> out[eoi].
+    // 8-channel rows are one 32-byte (fp16: 16-byte) store per lane.  Any other
+    // row goes through the warp's row buffer, and the warp then writes the 32
+    // rows' elements in memory order, 32 consecutive ones per store.  Stored
+    // from the accumulator's registers, one channel per instruction, a
+    // 9-channel row touched its sectors once per channel: 74.6M sector
+    // requests instead of about 10M on a 2160p frame, 1.49 GB through the
+    // SM-to-L2 crossbar instead of 0.3, and the decode took 345 us against 249
+    // with 8 channels (H = 64).  The buffer costs two shared-memory accesses
+    // per channel and nothing else waits on it.
+    float *rowbuf = reinterpret_cast<float *>(smem + tb.rows) +
+                    (size_t)(warp - NP * 4) * 32 * TmTables::row_words(C);
     auto out_rows = [&](uint32_t eoi, bool egood) {
       uint32_t o[16];
       tmem_ld16(tO + lanes, o);
       tmem_wait_ld();
       fence_before();
-      if (egood) {
-        // sigmoid(x) = 0.5 + 0.5 * tanh(x / 2)
+      auto sigmoid = [](uint32_t x) {  // 0.5 + 0.5 * tanh(x / 2)
+        float th;
+        asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * __uint_as_float(x)));
+        return fmaf(0.5f, th, 0.5f);
+      };
+      if (CP == 8 || ISS) {  // straight from the registers
+        if (!egood) return;
         float y[CP];
 #pragma unroll
-        for (int cc = 0; cc < CP; ++cc) {
-          float th;
-          asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * __uint_as_float(o[cc])));
-          y[cc] = fmaf(0.5f, th, 0.5f);
-        }
-        if (CP == 8 && vec_out && C == 8 && W.out_half) {  // one 16-byte store per row
+        for (int cc = 0; cc < CP; ++cc) y[cc] = sigmoid(o[cc]);
+        if (CP == 8 && tb.vector_rows && W.out_half) {  // one 16-byte store per row
           uint32_t h[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -667,7 +750,7 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
                                                                         (size_t)eoi * 8),
                        "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3])
                        : "memory");
-        } else if (CP == 8 && vec_out && C == 8) {  // one 32-byte store per row
+        } else if (CP == 8 && tb.vector_rows) {  // one 32-byte store per row
           asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(
                            reinterpret_cast<float *>(out) + (size_t)eoi * 8),
                        "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]), "f"(y[7])
@@ -677,7 +760,18 @@ __global__ void __launch_bounds__((NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 
           for (int cc = 0; cc < CP; ++cc)
             if (cc < (int)C) put_out(out, (size_t)eoi * C + cc, y[cc], W.out_half);
         }
+        return;
       }
+      const uint32_t S = TmTables::row_words(C);
+#pragma unroll
+      for (int cc = 0; cc < CP; ++cc)
+        if (cc < (int)C) rowbuf[lane * S + cc] = sigmoid(o[cc]);
+      __syncwarp();
+      if (W.out_half)
+        write_rows(reinterpret_cast<__half *>(out), rowbuf, C, eoi, egood, lane, tb.div_c);
+      else
+        write_rows(reinterpret_cast<float *>(out), rowbuf, C, eoi, egood, lane, tb.div_c);
+      __syncwarp();  // the next tile's rows overwrite the buffer
     };
     if constexpr (ISS) {
       // The epilogue warps of a consumer with issuer warps.  Per tile: A's
@@ -980,38 +1074,30 @@ cudaError_t launch_tm_t(const Assets &A, const WeightImages &W, const Buckets &B
                         unsigned long long *err, unsigned int *status, int num_sms, cudaStream_t st,
                         ntc_debug_row *dbg) {
   using M = TmSmem<H, NC, SC>;
-  const size_t smem = M::total;
+  // vector row stores need 8 channels and a base aligned to the row: 32 bytes
+  // (fp32) or 16 (fp16)
+  const bool vector_rows = W.out_dim == 8 && ((uintptr_t)out & (W.out_half ? 15 : 31)) == 0;
   const bool c8 = W.out_dim <= 8;
-  static PerDevice attr[2];
-  auto set_attrs = [&](auto kernel) {
-    return attr[c8].once([&]() {
-      // as little shared memory as the kernel needs: the rest of the array is L1
-      const int carve = (int)((smem * 100 + 232448 - 1) / 232448);
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
-      return e;
-    });
-  };
-  {
-    const cudaError_t e = c8 ? set_attrs(k_decode_tm<H, BF16, TRI, WRAP, 8, NP, NC, SC, DBG>)
-                             : set_attrs(k_decode_tm<H, BF16, TRI, WRAP, 16, NP, NC, SC, DBG>);
-    if (e != cudaSuccess) return e;
-  }
+  const uint32_t row_warps = issuer_warp<H>() || c8 ? 0 : NC * 4;  // consumer warps with a row buffer
+  const TmTables tb =
+      TmTables::plan(M::tables, A.num_sets * kLevels * A.num_mips, A.num_decoders, W.out_dim, vector_rows, row_warps);
   const size_t max_tiles = (n + kTile - 1) / kTile + A.num_decoders + 1;
   size_t grid = (size_t)num_sms;
   if (grid > max_tiles) grid = max_tiles;
-  // vector row stores need a base aligned to the row: 32 bytes (fp32) or 16 (fp16)
-  const int vec_out = ((uintptr_t)out & (W.out_half ? 15 : 31)) == 0;
   const unsigned threads = (NP + NC) * 128 + (issuer_warp<H>() ? NC * 64 : 0);
+  static PerDevice attr[2];
   // launched as a programmatic dependent of the bucketing: its prologue overlaps
   // the end of k_place
-  cudaError_t e;
-  if (c8)
-    e = launch_pdl(k_decode_tm<H, BF16, TRI, WRAP, 8, NP, NC, SC, DBG>, dim3((unsigned)grid), dim3(threads), smem, st,
-                   A, W, B, out, err, status, vec_out, dbg);
-  else
-    e = launch_pdl(k_decode_tm<H, BF16, TRI, WRAP, 16, NP, NC, SC, DBG>, dim3((unsigned)grid), dim3(threads), smem, st,
-                   A, W, B, out, err, status, vec_out, dbg);
+  auto launch = [&](auto kernel) {
+    const cudaError_t set = attr[c8].once([&]() {
+      const TmTables most = TmTables::plan(M::tables, kSmemGrids, kSmemTileTable - 2, 16, false, row_warps);
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most.total);
+    });
+    if (set != cudaSuccess) return set;
+    return launch_pdl_l1(kernel, dim3((unsigned)grid), dim3(threads), tb.total, st, A, W, B, out, err, status, tb, dbg);
+  };
+  const cudaError_t e = c8 ? launch(k_decode_tm<H, BF16, TRI, WRAP, 8, NP, NC, SC, DBG>)
+                           : launch(k_decode_tm<H, BF16, TRI, WRAP, 16, NP, NC, SC, DBG>);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

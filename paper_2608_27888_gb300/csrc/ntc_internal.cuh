@@ -644,21 +644,41 @@ class PerDevice {
 // replays one kernel of the chain needs it.
 bool pdl_enabled();
 
-// Launch with programmatic stream serialisation (see pdl_wait).
+// Launch with programmatic stream serialisation (see pdl_wait).  carve >= 0:
+// the share of the SM's array to set aside as shared memory, in percent.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                       Args... args) {
+cudaError_t launch_pdl_carve(int carve, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at[2];
+  unsigned k = 0;
+  if (pdl_enabled()) {
+    at[k].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[k++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (carve >= 0) {
+    at[k].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[k++].val.sharedMemCarveout = (unsigned)carve;
+  }
   cfg.attrs = at;
-  cfg.numAttrs = pdl_enabled() ? 1 : 0;
+  cfg.numAttrs = k;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  return launch_pdl_carve(-1, kernel, grid, block, smem, st, args...);
+}
+// One CTA per SM that takes as little of the array as its smem bytes need (and
+// the 1 KB the system keeps per CTA): the rest is L1.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_l1(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  constexpr size_t sm_bytes = 233472;
+  const int carve = (int)(((smem + 1024) * 100 + sm_bytes - 1) / sm_bytes);
+  return launch_pdl_carve(carve < 100 ? carve : 100, kernel, grid, block, smem, st, args...);
 }
 
 cudaError_t launch_build_pairs(const Assets &A, const uint32_t *chunk_grid, const uint32_t *chunk_start,
