@@ -4,13 +4,11 @@
 
 namespace ntc {
 
-size_t tc_image_bytes(uint32_t H) {
-  const size_t KH = H + 16;
-  return (size_t)H * kTcKA * 2 + (size_t)H * KH * 2 + (size_t)16 * KH * 2;
-}
+size_t tc_image_bytes(uint32_t H) { return pipe_image_bytes(kInDim, H, 2); }
 
 // One CTA per decoder: fp32 weights -> the shared-memory image of the tcgen05
-// kernel (bias folded in as column `in` of each layer's B operand).
+// kernel (each layer's bias, in kBiasParts parts, at the start of an extra
+// 16-wide K block).
 template <typename T>
 __global__ void k_pack_tc(const float *w32, uint32_t H, uint32_t C, uint8_t *tc, size_t tc_stride) {
   const uint32_t d = blockIdx.x;
@@ -18,27 +16,22 @@ __global__ void k_pack_tc(const float *w32, uint32_t H, uint32_t C, uint8_t *tc,
   const float *p = w32 + (size_t)d * P;
   const float *W1 = p, *b1 = W1 + H * 16, *W2 = b1 + H, *b2 = W2 + (size_t)H * H, *W3 = b2 + H,
               *b3 = W3 + (size_t)C * H;
-  const uint32_t KH = H + 16;
   uint8_t *img = tc + (size_t)d * tc_stride;
-  uint8_t *i1 = img, *i2 = i1 + (size_t)H * kTcKA * 2, *i3 = i2 + (size_t)H * KH * 2;
-  auto put = [](uint8_t *base, uint32_t r, uint32_t k, uint32_t K, float v) {
-    T h = T(v);
-    *reinterpret_cast<T *>(base + core_off(r, k, K)) = h;
+  // W [rows][in] and b [rows] (zeros beyond `real` rows) -> [rows][in + 16] at base
+  auto layer = [&](uint8_t *base, uint32_t rows, uint32_t real, uint32_t in, const float *W, const float *b) {
+    const uint32_t K = in + 16;
+    for (uint32_t i = threadIdx.x; i < rows * K; i += blockDim.x) {
+      const uint32_t r = i / K, k = i % K;
+      T v = T(0.0f);
+      if (r < real && k < in) v = T(W[(size_t)r * in + k]);
+      else if (r < real && k < in + kBiasParts) v = bias_part<T>(b[r], k - in);
+      *reinterpret_cast<T *>(base + core_off(r, k, K)) = v;
+    }
   };
-  for (uint32_t i = threadIdx.x; i < H * kTcKA; i += blockDim.x) {
-    uint32_t r = i / kTcKA, k = i % kTcKA;
-    put(i1, r, k, kTcKA, k < 16 ? W1[r * 16 + k] : (k == 16 ? b1[r] : 0.0f));
-  }
-  for (uint32_t i = threadIdx.x; i < H * KH; i += blockDim.x) {
-    uint32_t r = i / KH, k = i % KH;
-    put(i2, r, k, KH, k < H ? W2[(size_t)r * H + k] : (k == H ? b2[r] : 0.0f));
-  }
-  for (uint32_t i = threadIdx.x; i < 16 * KH; i += blockDim.x) {
-    uint32_t r = i / KH, k = i % KH;
-    float v = 0.0f;
-    if (r < C) v = k < H ? W3[(size_t)r * H + k] : (k == H ? b3[r] : 0.0f);
-    put(i3, r, k, KH, v);
-  }
+  uint8_t *i2 = img + (size_t)H * kTcKA * 2, *i3 = i2 + (size_t)H * (H + 16) * 2;
+  layer(img, H, H, 16, W1, b1);
+  layer(i2, H, H, H, W2, b2);
+  layer(i3, 16, C, H, W3, b3);
 }
 
 cudaError_t launch_pack_tc(const float *w32, uint32_t D, uint32_t H, uint32_t C, bool bf16,

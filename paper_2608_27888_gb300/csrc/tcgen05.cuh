@@ -77,10 +77,13 @@ __device__ __forceinline__ void wg_bar(int wg) {
   asm volatile("bar.sync %0, 128;\n" ::"r"(wg + 1) : "memory");
 }
 
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t K) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) |
-         ((uint64_t)(((K * 16u) >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+// Shared-memory descriptor of a no-swizzle K-major operand of K columns at
+// addr (16-byte aligned): K-adjacent core matrices 128 bytes apart, 8-row groups
+// K * 16 bytes apart.  16 more K columns: + 16 on the low word.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) {
+  return ((addr >> 4) & 0x3FFFu) | ((128u >> 4) << 16);
 }
+__device__ __forceinline__ uint32_t smem_desc_hi(uint32_t K) { return (K & 0x3FFFu) | (1u << 14); }
 
 template <bool BF16>
 __host__ __device__ constexpr uint32_t instr_desc(uint32_t N) {
@@ -135,13 +138,14 @@ __device__ __forceinline__ void tmem_wait_st() {
 }
 
 // D[tmem] (+)= A[tmem] x B[smem]: A read from tensor memory (row = lane, two
-// 16-bit K elements per 32-bit column).
-__device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
+// 16-bit K elements per 32-bit column).  B's descriptor comes as its two words:
+// the address field, the only one that changes, lies in the low one.
+__device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
                                         uint32_t accum) {
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b), "r"(idesc), "r"(accum)
+      "{\n.reg .pred p;\n.reg .b64 b;\nsetp.ne.b32 p, %5, 0;\nmov.b64 b, {%2, %3};\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accum)
       : "memory");
 }
 
