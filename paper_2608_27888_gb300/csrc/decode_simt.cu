@@ -13,96 +13,173 @@ __device__ __forceinline__ void count_bad(bool bad, unsigned long long *err) {
   if (m && (threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(err, (unsigned long long)__popc(m));
 }
 
-// fp32 decode: one 128-thread CTA per tile, one query per thread, the tile's
-// decoder in shared memory as fp32 (W1[H][16], b1, W2[H][H], b2, W3^T[H][CP],
-// b3[CP]).  Tiles are split into contiguous ranges per CTA so a CTA rarely
-// changes decoder.
+// fp32 decode over bucketed tiles: a CTA multiplies a tile's 128 activation
+// columns by its decoder's matrices out of shared memory, a thread 8 queries x
+// 8 outputs at a time, two queries per packed FMA.  Every sum runs over k in
+// increasing order from the bias, one rounding per term, as a scalar
+// evaluation would.  With one query per thread and the weights broadcast, each
+// 16-byte shared-memory read fed four FMAs and the reads were the bound (31
+// TFLOP/s on a 1080p frame, H = 64); here four of them feed 64.
+// Shared memory: W1^T [16][H], b1, W2^T [H][H], b2, W3^T [H][CP], b3[CP], the
+// activations [H][kActPitch] (feature columns first), the rows' output rows.
+// Tiles are split into contiguous ranges per CTA so a CTA rarely changes
+// decoder.
+constexpr int kActPitch = 132;  // 128 queries and a pad: 16-byte rows, stores of neighbouring rows on other banks
+
+template <int H>
+constexpr int fp32_threads() {
+  return (kTile / 8) * (H / 8);
+}
+
+__device__ __forceinline__ unsigned long long dup2(float x) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ void fma2(unsigned long long &acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+
+// acc[q pair][output] = b[output] + sum_k Wt[k][output] * act[k][query]; this
+// thread's queries are q0 .. q0 + 3 and q0 + 64 .. + 67, its outputs o0 .. o0 + 3
+// and o0 + H/2 .. + 3, so that a quarter warp's reads are one 128-byte row.
+template <int H, int K>
+__device__ __forceinline__ void fp32_layer(const float *Wt, const float *b, const float *act, int q0, int o0,
+                                           unsigned long long (&acc)[4][8]) {
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    const unsigned long long v = dup2(b[o0 + (o & 3) + (o >> 2) * (H / 2)]);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) acc[p][o] = v;
+  }
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) {
+    const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(act + k * kActPitch + q0);
+    const ulonglong2 a1 = *reinterpret_cast<const ulonglong2 *>(act + k * kActPitch + q0 + 64);
+    const float4 w0 = *reinterpret_cast<const float4 *>(Wt + k * H + o0);
+    const float4 w1 = *reinterpret_cast<const float4 *>(Wt + k * H + o0 + H / 2);
+    const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const unsigned long long ww = dup2(w[o]);
+      fma2(acc[0][o], ww, a0.x);
+      fma2(acc[1][o], ww, a0.y);
+      fma2(acc[2][o], ww, a1.x);
+      fma2(acc[3][o], ww, a1.y);
+    }
+  }
+}
+
+// ReLU of a layer's outputs into the activations
+template <int H>
+__device__ __forceinline__ void fp32_store(const unsigned long long (&acc)[4][8], float *act, int q0, int o0) {
+#pragma unroll
+  for (int o = 0; o < 8; ++o) {
+    float *r = act + (o0 + (o & 3) + (o >> 2) * (H / 2)) * kActPitch + q0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 x = unpack2(acc[2 * h][o]), y = unpack2(acc[2 * h + 1][o]);
+      *reinterpret_cast<float4 *>(r + 64 * h) =
+          make_float4(fmaxf(x.x, 0.0f), fmaxf(x.y, 0.0f), fmaxf(y.x, 0.0f), fmaxf(y.y, 0.0f));
+    }
+  }
+}
+
+inline __host__ __device__ size_t fp32_img_floats(uint32_t H, uint32_t C) { return (f32_image_floats(H, C) + 3) / 4 * 4; }
+inline __host__ __device__ size_t fp32_smem_bytes(uint32_t H, uint32_t C) {
+  return (fp32_img_floats(H, C) + (size_t)H * kActPitch + kTile) * 4;
+}
+
 template <int H, int CP>
-__global__ void __launch_bounds__(kTile) k_decode_fp32(Assets A, WeightImages W, Buckets B,
-                                                       float *out, unsigned long long *err) {
+__global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_fp32(Assets A, WeightImages W, Buckets B,
+                                                                                   float *out,
+                                                                                   unsigned long long *err) {
   extern __shared__ float4 smem4[];
   float *sw = reinterpret_cast<float *>(smem4);
-  const float *W1 = sw, *b1 = W1 + H * 16, *W2 = b1 + H, *b2 = W2 + H * H, *W3t = b2 + H,
-              *b3 = W3t + H * CP;
+  const float *W1 = sw, *b1 = W1 + H * 16, *W2 = b1 + H, *b2 = W2 + H * H, *W3t = b2 + H, *b3 = W3t + H * CP;
   const uint32_t D = A.num_decoders, C = W.out_dim;
+  float *act = sw + fp32_img_floats(H, C);
+  uint32_t *rows = reinterpret_cast<uint32_t *>(act + H * kActPitch);
+  constexpr uint32_t kNone = 0xFFFFFFFFu;  // never an output row
   const uint32_t T = __ldg(B.meta);
   const bool copied = rows_copied(B, D);
   const uint32_t t0 = (uint32_t)((unsigned long long)T * blockIdx.x / gridDim.x);
   const uint32_t t1 = (uint32_t)((unsigned long long)T * (blockIdx.x + 1) / gridDim.x);
   const size_t img_floats = f32_image_floats(H, C);
+  const int r = threadIdx.x & (kTile - 1);
+  const int q0 = ((threadIdx.x / 32 % 2) * 8 + threadIdx.x % 8) * 4, o0 = (threadIdx.x / 64 * 4 + threadIdx.x / 8 % 4) * 4;
   uint32_t cur = 0xFFFFFFFFu;
   for (uint32_t t = t0; t < t1; ++t) {
     uint32_t dec, start, len;
     tile_info(B.meta, D, t, dec, start, len);
+    __syncthreads();  // the previous tile has been written
     if (dec != cur && dec < D) {
-      __syncthreads();
       const float4 *src = reinterpret_cast<const float4 *>(W.f32 + (size_t)dec * W.f32_stride);
       for (uint32_t i = threadIdx.x; i < img_floats / 4; i += blockDim.x) smem4[i] = __ldg(src + i);
-      __syncthreads();
       cur = dec;
     }
-    const uint32_t r = threadIdx.x;
-    const bool valid = r < len;
-    ntc_query q;
-    uint32_t oi = 0;
-    bool bad = false;
-    if (valid) {
-      bucket_row(B, copied, start + r, oi, q);
-      bad = dec == D || query_bad(A, q);
-    }
-    count_bad(valid && bad, err);
-    if (!valid) continue;
-    float *o_row = out + (size_t)oi * C;
-    if (bad) {
-      for (uint32_t c = 0; c < C; ++c) o_row[c] = __int_as_float(0x7fc00000);
-      continue;
-    }
-    float f[kInDim];
-    query_features(A, q, f);
-    float h1[H];
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-      const float4 *w = reinterpret_cast<const float4 *>(W1 + j * 16);
-      float acc = b1[j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float4 x = w[i];
-        acc = fmaf(x.x, f[4 * i], acc);
-        acc = fmaf(x.y, f[4 * i + 1], acc);
-        acc = fmaf(x.z, f[4 * i + 2], acc);
-        acc = fmaf(x.w, f[4 * i + 3], acc);
+    if (threadIdx.x < kTile) {  // one query per thread: its features, or zeros
+      const bool valid = (uint32_t)r < len;
+      ntc_query q;
+      uint32_t oi = 0;
+      bool bad = false;
+      if (valid) {
+        bucket_row(B, copied, start + r, oi, q);
+        bad = dec == D || query_bad(A, q);
       }
-      h1[j] = fmaxf(acc, 0.0f);
-    }
-    float o[CP];
+      count_bad(valid && bad, err);
+      float f[kInDim];
 #pragma unroll
-    for (int c = 0; c < CP; ++c) o[c] = b3[c];
+      for (int k = 0; k < kInDim; ++k) f[k] = 0.0f;
+      if (valid && bad)
+        for (uint32_t c = 0; c < C; ++c) out[(size_t)oi * C + c] = __int_as_float(0x7fc00000);
+      if (valid && !bad) query_features(A, q, f);
+#pragma unroll
+      for (int k = 0; k < kInDim; ++k) act[k * kActPitch + r] = f[k];
+      rows[r] = valid && !bad ? oi : kNone;
+    }
+    if (dec >= D) continue;  // every row was bad
+    __syncthreads();
+    unsigned long long acc[4][8];
+    fp32_layer<H, kInDim>(W1, b1, act, q0, o0, acc);
+    __syncthreads();
+    fp32_store<H>(acc, act, q0, o0);
+    __syncthreads();
+    fp32_layer<H, H>(W2, b2, act, q0, o0, acc);
+    __syncthreads();
+    fp32_store<H>(acc, act, q0, o0);
+    __syncthreads();
+    // the output layer: a thread one query and CP outputs (H = 128: half of them)
+    constexpr int kO = CP * kTile / fp32_threads<H>();
+    const int c0 = (threadIdx.x / kTile) * kO;
+    float o[kO];
+#pragma unroll
+    for (int c = 0; c < kO; ++c) o[c] = b3[c0 + c];
 #pragma unroll 4
-    for (int j = 0; j < H; ++j) {
-      const float4 *w = reinterpret_cast<const float4 *>(W2 + j * H);
-      float acc = b2[j];
+    for (int k = 0; k < H; ++k) {
+      const float h = act[k * kActPitch + r];
+      const float4 *w3 = reinterpret_cast<const float4 *>(W3t + k * CP + c0);
 #pragma unroll
-      for (int i = 0; i < H / 4; ++i) {
-        float4 x = w[i];
-        acc = fmaf(x.x, h1[4 * i], acc);
-        acc = fmaf(x.y, h1[4 * i + 1], acc);
-        acc = fmaf(x.z, h1[4 * i + 2], acc);
-        acc = fmaf(x.w, h1[4 * i + 3], acc);
-      }
-      const float h = fmaxf(acc, 0.0f);
-      const float4 *w3 = reinterpret_cast<const float4 *>(W3t + j * CP);
-#pragma unroll
-      for (int i = 0; i < CP / 4; ++i) {
-        float4 x = w3[i];
+      for (int i = 0; i < kO / 4; ++i) {
+        const float4 x = w3[i];
         o[4 * i] = fmaf(x.x, h, o[4 * i]);
         o[4 * i + 1] = fmaf(x.y, h, o[4 * i + 1]);
         o[4 * i + 2] = fmaf(x.z, h, o[4 * i + 2]);
         o[4 * i + 3] = fmaf(x.w, h, o[4 * i + 3]);
       }
     }
+    const uint32_t oi = rows[r];
+    if (oi != kNone) {
+      float *o_row = out + (size_t)oi * C;
 #pragma unroll
-    for (int c = 0; c < CP; ++c)
-      if (c < (int)C) o_row[c] = 1.0f / (1.0f + expf(-o[c]));
+      for (int c = 0; c < kO; ++c)
+        if (c0 + c < (int)C) o_row[c0 + c] = 1.0f / (1.0f + expf(-o[c]));
+    }
   }
 }
 
@@ -210,12 +287,12 @@ __global__ void k_pack(const float *w32, uint32_t H, uint32_t C, uint8_t *mma, s
   float *f = f32 + (size_t)d * f32_stride;
   float *fW1 = f, *fb1 = fW1 + H * 16, *fW2 = fb1 + H, *fb2 = fW2 + (size_t)H * H, *fW3t = fb2 + H,
         *fb3 = fW3t + (size_t)H * CP;
-  for (uint32_t i = threadIdx.x; i < H * 16; i += blockDim.x) fW1[i] = W1[i];
+  for (uint32_t i = threadIdx.x; i < H * 16; i += blockDim.x) fW1[i] = W1[(i % H) * 16 + i / H];
   for (uint32_t i = threadIdx.x; i < H; i += blockDim.x) {
     fb1[i] = b1[i];
     fb2[i] = b2[i];
   }
-  for (uint32_t i = threadIdx.x; i < H * H; i += blockDim.x) fW2[i] = W2[i];
+  for (uint32_t i = threadIdx.x; i < H * H; i += blockDim.x) fW2[i] = W2[(size_t)(i % H) * H + i / H];
   for (uint32_t i = threadIdx.x; i < H * CP; i += blockDim.x) {
     uint32_t j = i / CP, c = i % CP;
     fW3t[i] = c < C ? W3[(size_t)c * H + j] : 0.0f;
@@ -226,17 +303,18 @@ __global__ void k_pack(const float *w32, uint32_t H, uint32_t C, uint8_t *mma, s
 template <int H, int CP>
 cudaError_t launch_fp32_t(const Assets &A, const WeightImages &W, const Buckets &B, size_t n,
                           float *out, unsigned long long *err, int num_sms, cudaStream_t st) {
-  const size_t smem = f32_image_floats(H, W.out_dim) * sizeof(float);
+  const size_t smem = fp32_smem_bytes(H, W.out_dim);
+  constexpr int threads = fp32_threads<H>();
   static PerDevice occ_of;
   const int occ = occ_of.value([&]() {
     cudaFuncSetAttribute(k_decode_fp32<H, CP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    const int o = resident_ctas(k_decode_fp32<H, CP>, kTile, smem);
+    const int o = resident_ctas(k_decode_fp32<H, CP>, threads, smem);
     return o < 1 ? 1 : o;
   });
   size_t max_tiles = (n + kTile - 1) / kTile + A.num_decoders + 1;
   size_t grid = (size_t)num_sms * occ;
   if (grid > max_tiles) grid = max_tiles;
-  k_decode_fp32<H, CP><<<(unsigned)grid, kTile, smem, st>>>(A, W, B, out, err);
+  k_decode_fp32<H, CP><<<(unsigned)grid, threads, smem, st>>>(A, W, B, out, err);
   return cudaGetLastError();
 }
 
