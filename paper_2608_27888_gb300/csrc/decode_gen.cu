@@ -40,30 +40,16 @@ __device__ __forceinline__ void produce_gen(const GenPipe<H, BF16, L * C> &pipe,
                                             const GridDesc *grids, void *out, unsigned long long *err) {
   constexpr int NF = L * C + 4 * kGenMaxPe;  // feature values this input layout can have
   constexpr int LW = L * C / 2, NW = (NF + 15) / 16 * 8;
-  const uint32_t D = A.num_decoders, K = pipe.K;
+  const uint32_t K = pipe.K;
   constexpr uint32_t NP = GenShape<H, L * C>::NP;
   const uint32_t p = (uint32_t)pipe.warp >> 2, row = threadIdx.x & 127;  // tiles p, p + NP, ...
-  const bool copied = rows_copied(B, D);
-  TileWalk walk;
-  // this thread's row of local tile k: its output row (kNoRow past the tile's
-  // end) and query record; the bad bucket (set id out of range) is rejected by
-  // query_bad().  The next tile's are loaded while tile k is gathered.
-  auto fetch_row = [&](uint32_t k, uint32_t &oi_, ntc_query &q_) {
-    oi_ = kNoRow;
-    if (k >= K) return;
-    uint32_t d_, st_, len_;
-    walk.at(pipe.seg, pipe.tst, D, pipe.tile(k), d_, st_, len_);
-    if (row < len_) bucket_row(B, copied, st_ + row, oi_, q_);
-  };
-  uint32_t oi;
-  ntc_query q;
-  fetch_row(p, oi, q);
+  typename GenPipe<H, BF16, L * C>::Rows rows(pipe, B, p);
   for (uint32_t k = p, j = 0; k < K && !pipe.wait.stopped(); k += NP, ++j) {
-    uint32_t noi;
-    ntc_query nq;
-    fetch_row(k + NP, noi, nq);
+    const ntc_query q = rows.record();
+    const uint32_t oi = rows.oi;
     const bool valid = oi != kNoRow;
     const bool good = valid && !query_bad(A, q);
+    rows.look_ahead(pipe, k, rows.oi);
     const bool bad = valid && !good;
     count_bad_warp(bad, err);
     if (bad) put_nan_row(out, oi, pipe.P.out_dim, pipe.P.out_half);
@@ -109,8 +95,6 @@ __device__ __forceinline__ void produce_gen(const GenPipe<H, BF16, L * C> &pipe,
       }
     }
     if (k < pipe.Kg) pipe.hand_over(p, j, k, row, pk, good ? oi : kNoRow);  // (a bad bucket's rows end here)
-    q = nq;
-    oi = noi;
   }
 }
 
@@ -277,7 +261,7 @@ cudaError_t launch_gen_tc_t(const Assets &A, const GenWeights &G, const Buckets 
   // weights arrive early (at H = 128 any number works: Pipe)
   uint32_t ns = 4;
   auto args = [&]() {
-    return pipe_args(G.tc, G.tc_stride, G.k1, H, G.layers, ns, stages, ngrids, A.num_decoders, G.out_dim, G.out_half, out);
+    return pipe_args(G.tc, G.tc_stride, G.k1, H, G.layers, ns, S::NP, stages, ngrids, A.num_decoders, G.out_dim, G.out_half, out, n);
   };
   PipeArgs P = args();
   while (ns > (H == 128 ? 1u : (uint32_t)S::T) && P.sm.total > (H == 128 ? kMostSmem : 131072u)) {

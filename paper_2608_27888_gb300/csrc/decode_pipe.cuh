@@ -53,18 +53,21 @@ constexpr uint32_t kBiasParts = 3;         // K columns of a bias block that car
 // what is left of the SM's array is the L1 that holds the gathers.
 struct PipeSmem {
   uint32_t img_pitch;  // weight images, one after another from 0
-  uint32_t oidx, bars, misc, grids, tiles, rows, total;
+  uint32_t oidx, recs, bars, misc, grids, tiles, rows, total;
   static __host__ __device__ __forceinline__ uint32_t row_words(uint32_t C) { return C | 1u; }  // no bank conflicts
-  static PipeSmem plan(uint32_t img_bytes, uint32_t ns, uint32_t ngrids, uint32_t D, uint32_t C, bool vector_rows) {
+  static PipeSmem plan(uint32_t img_bytes, uint32_t ns, uint32_t producers, uint32_t ngrids, uint32_t D, uint32_t C,
+                       bool row_buffer) {
     PipeSmem s;
     s.img_pitch = (img_bytes + 127) / 128 * 128;
     s.oidx = ns * s.img_pitch;
-    s.bars = s.oidx + kOidxRing * 128 * 4;
+    s.recs = s.oidx + kOidxRing * 128 * 4;
+    s.bars = s.recs + producers * 128 * (uint32_t)sizeof(ntc_query);
     s.misc = s.bars + 64 * 8;
     s.grids = s.misc + 128;
     s.tiles = s.grids + (ngrids <= kSmemGrids ? ngrids : 0u) * (uint32_t)sizeof(GridDesc);
     s.rows = s.tiles + (D + 2 <= kSmemTileTable ? 2 * (D + 2) : 0u) * 4;
-    s.total = s.rows + (vector_rows ? 0u : 4 * 32 * row_words(C) * 4);
+    // a row buffer per writer warp (its reads may run over by two rows of 32)
+    s.total = s.rows + (row_buffer ? (4 * 32 * row_words(C) + 64) * 4 : 0u);
     return s;
   }
 };
@@ -79,7 +82,8 @@ struct PipeArgs {
   uint32_t act, slope2;            // 0 ReLU, 1 LeakyReLU, 2 LeakyReLU with 0 <= slope <= 1 (slope2: in both halves)
   float slope;
   uint32_t out_dim, out_half;
-  uint32_t vector_rows, div_c;     // rows written as one vector store; k / C = k * div_c >> 16 for k < 512
+  uint32_t vector_rows;            // rows written as one vector store
+  uint32_t narrow;                 // every output element's index fits 32 bits
   PipeSmem sm;
 };
 
@@ -123,55 +127,78 @@ struct Waits {
 
 __device__ __forceinline__ void put_elem(float *p, float y) { *p = y; }
 __device__ __forceinline__ void put_elem(__half *p, float y) { *p = __float2half_rn(y); }
+// the same under a predicate: no branch, so that neighbouring elements overlap
+__device__ __forceinline__ void put_elem_if(bool on, float *p, float y) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.global.f32 [%0], %1;\n}\n" ::"l"(p), "f"(y),
+               "r"((uint32_t)on)
+               : "memory");
+}
+__device__ __forceinline__ void put_elem_if(bool on, __half *p, float y) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.global.u16 [%0], %1;\n}\n" ::"l"(p),
+               "h"(__half_as_ushort(__float2half_rn(y))), "r"((uint32_t)on)
+               : "memory");
+}
 
 // A warp's 32 output rows of C elements, from its row buffer (row r of the
 // warp at r * PipeSmem::row_words(C)) to out: element k = lane + 32 i of the
 // 32 x C block in store i, so that a store covers consecutive elements of a few
-// rows.  One channel per store instead touches each sector of a row once per
-// channel: for 9 channels 74.6M sector requests on a 2160p frame, 1.49 GB
-// through the SM-to-L2 crossbar instead of 0.3.
-template <typename E>
-__device__ __forceinline__ void write_rows(E *out, const float *rowbuf, uint32_t C, uint32_t oi, bool good, int lane,
-                                           uint32_t div_c) {
-  const uint32_t oi0 = __shfl_sync(0xFFFFFFFFu, oi, 0);
-  const bool side_by_side = __all_sync(0xFFFFFFFFu, good && oi == oi0 + (uint32_t)lane);
-  if (side_by_side && (C & 1)) {  // the block is 32 C consecutive elements on both sides
-    E *p = out + (size_t)oi0 * C + lane;
-    const float *b = rowbuf + lane;
+// rows.  Stored straight from the accumulator instead, one channel per
+// instruction, a nine-channel row's sectors are touched once per channel, 1.5 GB
+// through the SM-to-L2 crossbar for a 2160p frame instead of 0.3; but each
+// shared-memory or shuffle step of this way queues behind the producers'
+// gathers.  At H = 128 the crossbar is what matters (four trilinear 2160p
+// frames: decode 1,410 -> 1,341 us with the buffer), at H = 64 the writers'
+// time per tile (2160p frame 295 us with it, 228 without; Sec. 4's decoder on
+// 1080p 116 and 82).
+struct RowWriter {
+  uint32_t at[16];  // element i: its row in the low 5 bits, its channel from bit 8
+  __device__ __forceinline__ RowWriter(uint32_t C, int lane) {
+#pragma unroll
+    for (uint32_t i = 0; i < 16; ++i) {
+      const uint32_t k = (uint32_t)lane + 32 * i, r = k / C;
+      at[i] = (r & 31u) | (k - r * C) << 8;
+    }
+  }
+  // narrow: every element's index fits 32 bits
+  template <typename E>
+  __device__ __forceinline__ void operator()(E *out, const float *rowbuf, uint32_t C, uint32_t oi, bool good, int lane,
+                                             bool narrow) const {
+    const uint32_t oi0 = __shfl_sync(0xFFFFFFFFu, oi, 0);
+    if ((C & 1) && __all_sync(0xFFFFFFFFu, good && oi == oi0 + (uint32_t)lane)) {
+      // the rows are side by side: 32 C consecutive elements on both sides
+      E *p = out + (size_t)oi0 * C + lane;
+#pragma unroll
+      for (uint32_t g = 0; g < 16; g += 3) {
+        if (g >= C) break;
+        float v[3];
+#pragma unroll
+        for (uint32_t j = 0; j < 3; ++j) v[j] = rowbuf[lane + 32 * (g + j)];
+#pragma unroll
+        for (uint32_t j = 0; j < 3; ++j) put_elem_if(g + j < C, p + 32 * (g + j), v[j]);
+      }
+      return;
+    }
+    const uint32_t even = 1u - (C & 1u);
+    const uint32_t base = good ? (narrow ? oi * C : oi) : kNoRow;  // the row's first element, or the row
 #pragma unroll
     for (uint32_t g = 0; g < 16; g += 3) {
       if (g >= C) break;
       float v[3];
+      uint32_t to[3];
 #pragma unroll
-      for (uint32_t j = 0; j < 3; ++j)
-        if (g + j < C) v[j] = b[32 * (g + j)];
+      for (uint32_t j = 0; j < 3; ++j) {
+        const uint32_t i = g + j < 16 ? g + j : 15, w = at[i];
+        to[j] = __shfl_sync(0xFFFFFFFFu, base, w);
+        v[j] = rowbuf[(uint32_t)lane + 32 * i + even * (w & 31u)];
+      }
 #pragma unroll
-      for (uint32_t j = 0; j < 3; ++j)
-        if (g + j < C) put_elem(p + 32 * (g + j), v[j]);
+      for (uint32_t j = 0; j < 3; ++j) {
+        const uint32_t i = g + j < 16 ? g + j : 15, ch = at[i] >> 8;
+        put_elem_if(g + j < C && to[j] != kNoRow, out + (narrow ? (size_t)(to[j] + ch) : (size_t)to[j] * C + ch), v[j]);
+      }
     }
-    return;
   }
-  const uint32_t row = good ? oi : kNoRow, even = 1u - (C & 1u);
-#pragma unroll
-  for (uint32_t g = 0; g < 16; g += 3) {
-    if (g >= C) break;
-    float v[3];
-    uint32_t ro[3], ch[3];
-#pragma unroll
-    for (uint32_t j = 0; j < 3; ++j) {
-      const uint32_t k = (uint32_t)lane + 32 * (g + j), r = k * div_c >> 16;
-      ch[j] = k - r * C;
-      ro[j] = __shfl_sync(0xFFFFFFFFu, row, r & 31u);
-      if (g + j < C)
-        v[j] = rowbuf[k + even * r];
-      else
-        ro[j] = kNoRow;
-    }
-#pragma unroll
-    for (uint32_t j = 0; j < 3; ++j)
-      if (ro[j] != kNoRow) put_elem(out + (size_t)ro[j] * C + ch[j], v[j]);
-  }
-}
+};
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
@@ -355,6 +382,64 @@ struct Pipe {
     K = local(all);
     Kg = local(good);
   }
+
+  // The rows of one producer thread, tile by tile (k = p, p + NP, ...): while
+  // tile k is gathered, the record of its next tile is on its way to the
+  // thread's slot in shared memory (cp.async: no registers) and the output row
+  // (perm) of the one after it to a register, so that neither a record nor the
+  // perm entry that leads to it is waited for.  Loaded one tile ahead together,
+  // they cost a 1080p frame's producers about a quarter of their time.
+  struct Rows {
+    const Buckets &B;
+    TileWalk walk;
+    bool copied;
+    uint32_t slot;       // shared memory of this thread's record
+    uint32_t oi;         // output row of the current tile, or kNoRow past its end
+    uint32_t noi, npos;  // of the next tile, and its place in bucket order
+    // a row of the bad bucket (set id out of range) needs no flag of its own:
+    // query_bad() rejects it
+    __device__ __forceinline__ void row_of(const Pipe &q, uint32_t k, uint32_t &oi_, uint32_t &pos) {
+      oi_ = kNoRow;
+      if (k >= q.K) return;
+      uint32_t d, st, len;
+      const uint32_t row = threadIdx.x & 127;
+      walk.at(q.seg, q.tst, q.D_, q.tile(k), d, st, len);
+      if (row >= len) return;
+      pos = st + row;
+      oi_ = q.ident_n ? pos : __ldg(B.perm + pos);
+    }
+    __device__ __forceinline__ void request() {  // the next tile's record
+      if (noi != kNoRow)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(slot),
+                     "l"(copied ? B.sorted + npos : B.queries + noi)
+                     : "memory");
+    }
+    __device__ __forceinline__ Rows(const Pipe &q, const Buckets &b, uint32_t p) : B(b) {
+      walk.ident_n = q.ident_n;
+      copied = rows_copied(B, q.D_);
+      slot = q.sbase + q.P.sm.recs + (p * 128 + (threadIdx.x & 127)) * (uint32_t)sizeof(ntc_query);
+      row_of(q, p, noi, npos);
+      request();
+      oi = noi;
+      row_of(q, p + NP, noi, npos);
+    }
+    // the current tile's record (undefined past the tile's end)
+    __device__ __forceinline__ ntc_query record() const {
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+      ntc_query r;
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];\n"
+                   : "=r"(r.set_id), "=f"(r.u), "=f"(r.v), "=f"(r.lod)
+                   : "r"(slot)
+                   : "memory");
+      return r;
+    }
+    // after record() of tile k has been looked at
+    __device__ __forceinline__ void look_ahead(const Pipe &q, uint32_t k, uint32_t &next) {
+      request();
+      next = noi;
+      row_of(q, k + 2 * NP, noi, npos);
+    }
+  };
 
   // Ends the CTA: every role has left.
   __device__ __forceinline__ void end() const {
@@ -564,6 +649,7 @@ struct Pipe {
   __device__ __forceinline__ void writer(void *out) const {
     const uint32_t row = threadIdx.x & 127, C = P.out_dim;
     float *rowbuf = reinterpret_cast<float *>(smem + P.sm.rows) + (warp & 3) * 32 * PipeSmem::row_words(C);
+    const RowWriter write(kRowBuffer ? C : 16u, lane);
     auto sigmoid = [](uint32_t x) {  // 0.5 + 0.5 * tanh(x / 2)
       float th;
       asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * __uint_as_float(x)));
@@ -605,18 +691,37 @@ struct Pipe {
         }
         continue;
       }
-      const uint32_t S = PipeSmem::row_words(C);
+      if (!kRowBuffer) {
+        if (good)
 #pragma unroll
-      for (int c = 0; c < 16; ++c)
-        if (c < (int)C) rowbuf[lane * S + c] = sigmoid(o[c]);
+          for (int c = 0; c < 16; ++c)
+            if (c < (int)C) put_out(out, (size_t)oi * C + c, sigmoid(o[c]), P.out_half);
+        continue;
+      }
+      const uint32_t row_at = saddr(rowbuf) + lane * PipeSmem::row_words(C) * 4;
+#pragma unroll
+      for (int h = 0; h < 16; h += 8) {
+        if (h >= (int)C) break;
+        float y[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) y[c] = sigmoid(o[h + c]);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          asm volatile("{\n.reg .pred p;\nsetp.lt.u32 p, %2, %3;\n@p st.shared.f32 [%0], %1;\n}\n" ::"r"(
+                           row_at + (h + c) * 4),
+                       "f"(y[c]), "r"((uint32_t)(h + c)), "r"(C)
+                       : "memory");
+      }
       __syncwarp();
       if (P.out_half)
-        write_rows(reinterpret_cast<__half *>(out), rowbuf, C, oi, good, lane, P.div_c);
+        write(reinterpret_cast<__half *>(out), rowbuf, C, oi, good, lane, P.narrow != 0);
       else
-        write_rows(reinterpret_cast<float *>(out), rowbuf, C, oi, good, lane, P.div_c);
+        write(reinterpret_cast<float *>(out), rowbuf, C, oi, good, lane, P.narrow != 0);
       __syncwarp();  // the next tile's rows overwrite the buffer
     }
   }
+
+  static constexpr bool kRowBuffer = H == 128;
 
   // The roles other than the producers.
   __device__ __forceinline__ void consume(void *out) const {
@@ -652,8 +757,8 @@ __device__ __forceinline__ T bias_part(float b, uint32_t j) {
 
 // The launch arguments that both decodes derive alike.
 inline PipeArgs pipe_args(const uint8_t *img, size_t stride, uint32_t k1, uint32_t hidden, uint32_t layers, uint32_t ns,
-                          uint32_t stages, uint32_t ngrids, uint32_t decoders, uint32_t out_dim, uint32_t out_half,
-                          const void *out) {
+                          uint32_t producers, uint32_t stages, uint32_t ngrids, uint32_t decoders, uint32_t out_dim, uint32_t out_half,
+                          const void *out, size_t n) {
   PipeArgs P{};
   P.img = img;
   P.img_stride = stride;
@@ -667,8 +772,8 @@ inline PipeArgs pipe_args(const uint8_t *img, size_t stride, uint32_t k1, uint32
   // vector row stores need 8 channels and a base aligned to the row: 32 bytes
   // (fp32) or 16 (fp16)
   P.vector_rows = out_dim == 8 && ((uintptr_t)out & (out_half ? 15 : 31)) == 0;
-  P.div_c = (65536 + out_dim - 1) / out_dim;
-  P.sm = PipeSmem::plan(P.img_bytes, ns, ngrids, decoders, out_dim, P.vector_rows);
+  P.narrow = (unsigned long long)n * out_dim < 0xFFFFFFFFull;
+  P.sm = PipeSmem::plan(P.img_bytes, ns, producers, ngrids, decoders, out_dim, hidden == 128 && !P.vector_rows);
   return P;
 }
 

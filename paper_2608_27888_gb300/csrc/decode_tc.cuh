@@ -201,64 +201,16 @@ __device__ __forceinline__ void produce_tm(const TmPipe<H, BF16> &pipe, const As
                                            const GridDesc *grids, void *out, unsigned long long *err,
                                            ntc_debug_row *dbg) {
   constexpr uint32_t NP = TmShape<H>::NP;
-  const uint32_t D = A.num_decoders, K = pipe.K;
+  const uint32_t K = pipe.K;
   const uint32_t p = (uint32_t)pipe.warp >> 2, row = threadIdx.x & 127;  // tiles p, p + NP, ...
   const int lane = pipe.lane;
-  // Records read through perm (the caller's array, when the bucketing did not
-  // copy them): the output rows are loaded two tiles ahead and the query
-  // records one tile ahead, so a record never waits on its own perm load (DEEP;
-  // the H = 64 kernels that blend mips have no registers to spare for it).
-  // Otherwise a row's output row and record are loaded together, one tile
-  // ahead.
-  constexpr bool DEEP = H > 64 || !TRI;
-  const bool copied = rows_copied(B, D);
-  const bool two_stage = DEEP && !copied;
-  TileWalk walk;
-  walk.ident_n = B.identity_n;
-  // this thread's row of local tile k: its output row, or kNoRow past the
-  // tile's end.  A row of the bad bucket (set id out of range) needs no flag of
-  // its own: query_bad() rejects it.
-  auto out_row = [&](uint32_t k) -> uint32_t {
-    if (k >= K) return kNoRow;
-    uint32_t d_, st_, len_;
-    walk.at(pipe.seg, pipe.tst, D, pipe.tile(k), d_, st_, len_);
-    if (row >= len_) return kNoRow;
-    return B.identity_n ? st_ + row : __ldg(B.perm + st_ + row);
-  };
-  // one stage: the row's output row and query record together
-  auto fetch_row = [&](uint32_t k, uint32_t &oi_, ntc_query &q_) {
-    oi_ = kNoRow;
-    if (k >= K) return;
-    uint32_t d_, st_, len_;
-    walk.at(pipe.seg, pipe.tst, D, pipe.tile(k), d_, st_, len_);
-    if (row < len_) bucket_row(B, copied, st_ + row, oi_, q_);
-  };
-  uint32_t oi, noi = kNoRow;
-  ntc_query q;
-  if (two_stage) {
-    oi = out_row(p);
-    noi = out_row(p + NP);
-    if (oi != kNoRow) q = load_query(B.queries + oi);
-  } else {
-    fetch_row(p, oi, q);
-  }
+  typename TmPipe<H, BF16>::Rows rows(pipe, B, p);
   for (uint32_t k = p, j = 0; k < K && !pipe.wait.stopped(); k += NP, ++j) {
-    // the next tile's query record (and, two-stage, the output row of the
-    // tile after it) go in flight early: before the taps, or (TRI, where
-    // registers are scarcer) once the first mip's taps are consumed
-    uint32_t nnoi = kNoRow;
-    ntc_query nq;
-    auto prefetch = [&]() {
-      if (two_stage) {
-        if (noi != kNoRow) nq = load_query(B.queries + noi);
-        nnoi = out_row(k + 2 * NP);
-      } else {
-        fetch_row(k + NP, noi, nq);
-      }
-    };
-    if (!TRI) prefetch();
+    const ntc_query q = rows.record();
+    const uint32_t oi = rows.oi;
     const bool valid = oi != kNoRow;
     const bool good = valid && !query_bad(A, q);
+    rows.look_ahead(pipe, k, rows.oi);
     Taps taps;
     MipPick mp;
     TapIdx ti[kLevels];
@@ -296,7 +248,6 @@ __device__ __forceinline__ void produce_tm(const TmPipe<H, BF16> &pipe, const As
     if (bad) put_nan_row(out, oi, pipe.P.out_dim, pipe.P.out_half);
     __half2 acc[kLevels][4];
     accum_taps<true>(taps, acc);
-    if (TRI) prefetch();
     if (TRI && __any_sync(0xFFFFFFFFu, good && mp.t > 0.0f)) {  // some row blends two mips
 #pragma unroll
       for (int lv = 0; lv < kLevels; ++lv) {
@@ -315,9 +266,6 @@ __device__ __forceinline__ void produce_tm(const TmPipe<H, BF16> &pipe, const As
 #pragma unroll
       for (int i = 0; i < 8; ++i) dbg[oi].feat[i] = a[i];
     if (k < pipe.Kg) pipe.hand_over(p, j, k, row, a, good ? oi : kNoRow);  // (a bad bucket's rows end here)
-    q = nq;
-    oi = noi;
-    if (two_stage) noi = nnoi;
   }
 }
 
@@ -340,13 +288,13 @@ cudaError_t launch_tm_t(const Assets &A, const WeightImages &W, const Buckets &B
                         unsigned long long *err, unsigned int *status, int num_sms, cudaStream_t st,
                         ntc_debug_row *dbg) {
   using S = TmShape<H>;
-  const PipeArgs P = pipe_args(W.tc, W.tc_stride, kInDim, H, 2, S::IMAGES, S::NP, A.num_sets * kLevels * A.num_mips,
-                               A.num_decoders, W.out_dim, W.out_half, out);
+  const PipeArgs P = pipe_args(W.tc, W.tc_stride, kInDim, H, 2, S::IMAGES, S::NP, S::NP, A.num_sets * kLevels * A.num_mips,
+                               A.num_decoders, W.out_dim, W.out_half, out, n);
   static_assert(pipe_columns(H, S::T, kInDim, S::NP) <= 512, "tensor memory plan exceeds 512 columns");
   const auto kernel = k_decode_tm<H, BF16, TRI, WRAP, DBG>;
   static PerDevice attr;
   cudaError_t e = attr.once([&]() {
-    const PipeSmem most = PipeSmem::plan(P.img_bytes, S::IMAGES, kSmemGrids, kSmemTileTable - 2, 16, false);
+    const PipeSmem most = PipeSmem::plan(P.img_bytes, S::IMAGES, S::NP, kSmemGrids, kSmemTileTable - 2, 16, true);
     return allow_smem((const void *)kernel, most.total);
   });
   if (e != cudaSuccess) return e;

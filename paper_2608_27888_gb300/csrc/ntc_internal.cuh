@@ -456,10 +456,6 @@ __device__ __forceinline__ void tile_info(const uint32_t *meta, uint32_t D, uint
   len = min((uint32_t)kTile, end - start);
 }
 
-// The tiles of one role in increasing order: the decoder index only moves
-// forward, so a lookup is a few compares instead of a binary search.  With
-// ident_n != 0 (one decoder, nothing sorted) tile t is queries 128t .. of the
-// caller's array.
 // One output value in the context's output format: fp32, or IEEE half rounded
 // to nearest even (the fp16 output of Sec. 4.4's fp16 kernels); a bad query's
 // row is NaN in every channel.
@@ -478,9 +474,16 @@ __device__ __forceinline__ void put_nan_row(void *out, size_t row, uint32_t C, b
   }
 }
 
+// The tiles of one role in increasing order: the decoder index only moves
+// forward, so a lookup is a few compares instead of a binary search.  With
+// ident_n != 0 (one decoder, nothing sorted) tile t is queries 128t .. of the
+// caller's array.
 struct TileWalk {
   uint32_t d = 0;
   uint32_t ident_n = 0;
+  // of decoder d, once looked up: its first tile after, and its queries' end;
+  // tile t starts at base + t * kTile
+  uint32_t next = 0, end = 0, base = 0;
   __device__ __forceinline__ void at(const uint32_t *seg, const uint32_t *tst, uint32_t D, uint32_t t,
                                      uint32_t &dec, uint32_t &start, uint32_t &len) {
     if (ident_n) {
@@ -489,10 +492,15 @@ struct TileWalk {
       len = min((uint32_t)kTile, ident_n - start);
       return;
     }
-    while (d < D && tst[d + 1] <= t) ++d;
+    if (t >= next) {  // another decoder (next = 0: the first call)
+      while (d < D && tst[d + 1] <= t) ++d;
+      next = d < D ? tst[d + 1] : 0xFFFFFFFFu;
+      end = seg[d + 1];
+      base = seg[d] - tst[d] * kTile;
+    }
     dec = d;
-    start = seg[d] + (t - tst[d]) * kTile;
-    len = min((uint32_t)kTile, seg[d + 1] - start);
+    start = base + t * kTile;
+    len = min((uint32_t)kTile, end - start);
   }
 };
 
