@@ -41,7 +41,7 @@
  * range or whose u or v is not finite decodes to NaN in every channel and is
  * counted (ntc_get_error_count).  No kernel traps.
  *
- * Environment: the bucketing kernels and the tensor-core decode after them
+ * Environment: the bucketing kernels and the tensor-core decodes after them
  * are launched as programmatic dependents of their predecessor on the stream
  * (each starts while the one before is finishing and waits for its results).
  * With NTC_NO_PDL set (any value, read once per process) they are ordinary
@@ -298,7 +298,8 @@ NTC_API size_t ntc_max_tiles(const ntc_ctx *ctx, size_t n);
  * counterpart: the paper's queries are always valid).  Synchronises
  * the device.  Returns NTC_ERR_CUDA (and still writes *count) when a kernel
  * gave up one of its bounded waits since then (every mbarrier wait of the
- * tcgen05 kernels ends after 200 ms; the bucketing waits on nothing): that
+ * tcgen05 kernels ends after 200 ms; the bucketing waits on nothing but, in
+ * calls of up to 65,536 queries, a hardware cluster barrier): that
  * call's results are invalid, the context stays usable.  The reset clears
  * both. */
 NTC_API ntc_status ntc_get_error_count(ntc_ctx *ctx, uint64_t *count);

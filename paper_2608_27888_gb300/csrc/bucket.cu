@@ -4,7 +4,7 @@
 // the queries of one block; sorting the queries by decoder (stable, so each
 // bucket keeps the original order) turns the interleaved stream into runs of
 // single-decoder 128-query tiles.  Three kernels, none of which waits for
-// another CTA:
+// another CTA of its own:
 //   k_count  per 2048-query chunk: every query's decoder (set -> decoder map;
 //            out-of-range set ids form the extra bucket D), written as one
 //            byte (two beyond 255 decoders), the chunk's count of every
@@ -31,6 +31,7 @@
 // contiguous records.  Equal decoders within a warp are found with one ballot
 // per bit of the decoder id.  The permutation is exactly std::stable_sort of
 // the indices by decoder.
+// Calls of up to 65,536 queries take one launch instead (k_bucket_small).
 #include <algorithm>
 
 #include "ntc_internal.cuh"
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_count(Assets A, const ntc_qu
   const size_t wbase = (size_t)blockIdx.x * kBucketChunk + (size_t)warp * (kBucketItems * 32);
   const uint32_t *sid = reinterpret_cast<const uint32_t *>(q);
   uint32_t s[kBucketItems];
+  pdl_wait();  // whatever wrote the queries, and the last reader of the scratch
 #pragma unroll
   for (int it = 0; it < kBucketItems; ++it) {  // every load in flight before any is used
     const size_t j = wbase + it * 32 + lane;
@@ -456,6 +458,167 @@ __global__ void __launch_bounds__(kBucketThreads, 5) k_place(Assets A, const ntc
   }
 }
 
+// ------------------------------------------------------------ small calls
+
+// The whole bucketing of up to kSmallMax queries in one launch, by one cluster
+// of up to 16 CTAs (the cluster barrier is the only wait).  A CTA takes
+// `items` x 1024 consecutive queries, a warp `items` x 32 of them: it keeps their
+// decoders in shared memory and counts them, a shuffle scan per decoder turns
+// the warps' counts into offsets, the CTAs read each other's totals through
+// distributed shared memory, and every warp then places its own run with no
+// further barrier.  Same permutation, tile table and copy decision as the three
+// kernels above, which cost about 16 us of chained launches whatever the size.
+// A whole decode call, with them and this way: 1,000 queries of 16 decoders
+// 20.5 -> 11.2 us, 32,000 20.6 -> 15.5, 65,536 22.6 -> 19.6 (and, by issue on so
+// few SMs, 131,072 24.7 -> 37 with 8 CTAs: hence the limit).
+constexpr uint32_t kSmallThreads = 1024, kSmallWarps = 32, kSmallCtas = 16, kSmallItems = 4;
+constexpr size_t kSmallMax = (size_t)kSmallCtas * kSmallThreads * kSmallItems;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+// *p of CTA `rank` of the cluster, p in shared memory
+__device__ __forceinline__ uint32_t cluster_read(const uint32_t *p, uint32_t rank) {
+  uint32_t v;
+  asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %1, %2;\nld.shared::cluster.u32 %0, [a];\n}\n"
+               : "=r"(v)
+               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank)
+               : "memory");
+  return v;
+}
+
+constexpr int kSmallSmem = 200 * 1024;  // dynamic shared memory of a CTA, at most
+inline size_t small_smem_bytes(uint32_t D, uint32_t items) {
+  return ((size_t)kSmallWarps + 4) * (D + 2) * 4 + (size_t)kSmallThreads * items * 2;
+}
+
+__global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const ntc_query *q, uint32_t n, uint32_t items,
+                                                                uint32_t *meta, uint32_t *perm, ntc_query *sorted) {
+  // shared memory: per-warp counters [32][D+2]; per decoder the CTA's total,
+  // its place of the CTA's first query, and the scans [D+2] each; the decoders
+  // of the CTA's queries [1024 x items]
+  extern __shared__ uint32_t small_sm[];
+  __shared__ uint32_t ws[32];
+  __shared__ uint32_t s_div;
+  const uint32_t D = A.num_decoders, DW = D + 2;
+  uint32_t *cnt = small_sm, *tot = cnt + kSmallWarps * DW, *gbase = tot + DW, *seg = gbase + DW, *tst = seg + DW;
+  uint16_t *keys = reinterpret_cast<uint16_t *>(tst + DW);
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = cluster_rank(), ctas = cluster_size();
+  for (uint32_t i = threadIdx.x; i < kSmallWarps * DW; i += kSmallThreads) cnt[i] = 0;
+  if (threadIdx.x == 0) s_div = 0;
+  const MapLookup lookup(A);
+  const int nbits = key_bits(D);
+  __syncthreads();
+  pdl_wait();     // whatever wrote the queries
+  pdl_trigger();  // the decode may launch (it waits for this grid before reading)
+  const uint32_t run = warp * items * 32;                         // this warp's run in the CTA's queries
+  const uint32_t first = rank * items * kSmallThreads + run;      // and in the call's
+  const uint32_t *sid = reinterpret_cast<const uint32_t *>(q);
+  uint32_t *my = cnt + warp * DW;
+  uint32_t div = 0;
+  for (uint32_t it = 0; it < items && first + it * 32 < n; it += 8) {
+    uint32_t s[8];
+#pragma unroll
+    for (uint32_t u = 0; u < 8; ++u) {  // eight loads in flight
+      const uint32_t j = first + (it + u) * 32 + lane;
+      s[u] = it + u < items && j < n ? __ldg(sid + 4 * (size_t)j) : 0u;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < 8; ++u) s[u] = lookup(A, s[u]);  // every lane: the lookup shuffles
+    for (uint32_t u = 0; u < 8 && it + u < items; ++u) {
+      uint32_t d = s[0];
+#pragma unroll
+      for (uint32_t v = 1; v < 8; ++v) d = u == v ? s[v] : d;
+      if (first + (it + u) * 32 + lane >= n) d = D + 1;  // no query
+      keys[run + (it + u) * 32 + lane] = (uint16_t)d;
+      const uint32_t m = match_key(d, nbits);
+      const bool leader = lane == (uint32_t)__ffs(m) - 1;
+      if (leader) my[d] += __popc(m);
+      const uint32_t runs = __popc(__ballot_sync(0xFFFFFFFFu, leader && d <= D));
+      div += runs ? runs - 1 : 0u;
+      __syncwarp();
+    }
+  }
+  // runs past the end: no queries
+  for (uint32_t it = 0; it < items; ++it)
+    if (first + it * 32 >= n) keys[run + it * 32 + lane] = (uint16_t)(D + 1);
+  if (lane == 0 && div) atomicAdd(&s_div, div);
+  __syncthreads();
+  for (uint32_t d = warp; d <= D; d += kSmallWarps) {  // the warps' counts of decoder d -> offsets
+    const uint32_t x = cnt[lane * DW + d];
+    uint32_t y = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_up_sync(0xFFFFFFFFu, y, o);
+      if (lane >= (uint32_t)o) y += z;
+    }
+    cnt[lane * DW + d] = y - x;
+    if (lane == 31) tot[d] = y;
+  }
+  cluster_arrive();
+  cluster_wait();
+  uint32_t all_div = 0;
+  for (uint32_t d = threadIdx.x; d <= D; d += kSmallThreads) {
+    uint32_t before = 0, total = 0;
+    for (uint32_t r = 0; r < ctas; ++r) {
+      const uint32_t v = cluster_read(tot + d, r);
+      before += r < rank ? v : 0u;
+      total += v;
+    }
+    gbase[d] = before;
+    seg[d] = total;
+    tst[d] = (total + kTile - 1) / kTile;
+  }
+  for (uint32_t r = 0; r < ctas; ++r) all_div += cluster_read(&s_div, r);
+  cluster_arrive();  // (waited for before leaving: no CTA's shared memory goes while others read it)
+  __syncthreads();
+  block_scan_to(seg, seg, D + 1, ws);
+  __syncthreads();
+  const bool copy = (uint64_t)all_div > (uint64_t)kCopyAboveScore * ((n + 31) / 32);
+  if (rank == 0) {
+    const uint32_t nt = block_scan_to(tst, tst, D + 1, ws);
+    __syncthreads();
+    for (uint32_t d = threadIdx.x; d <= D; d += kSmallThreads) {
+      meta[1 + d] = seg[d];
+      meta[1 + DW + d] = tst[d];
+    }
+    if (threadIdx.x == 0) {
+      meta[0] = nt;
+      meta[1 + D + 1] = n;
+      meta[1 + DW + D + 1] = nt;
+      meta[meta_copied(D)] = copy;
+      meta[meta_divergence(D)] = all_div;
+    }
+  }
+  const uint32_t lt = (1u << lane) - 1u;
+  for (uint32_t it = 0; it < items && first + it * 32 < n; ++it) {
+    const uint32_t d = keys[run + it * 32 + lane], j = first + it * 32 + lane;
+    const uint32_t m = match_key(d, nbits);
+    const uint32_t at = my[d] + __popc(m & lt);
+    __syncwarp();
+    if (lane == (uint32_t)__ffs(m) - 1) my[d] += __popc(m);
+    __syncwarp();
+    if (d > D) continue;
+    const uint32_t p = seg[d] + gbase[d] + at;
+    if (p < n) {
+      perm[p] = j;
+      if (copy) reinterpret_cast<uint4 *>(sorted)[p] = __ldg(reinterpret_cast<const uint4 *>(q + j));
+    }
+  }
+  cluster_wait();
+}
+
 __global__ void k_tiles_export(const uint32_t *meta, uint32_t D, uint32_t *tiles, uint32_t *num_tiles,
                                uint32_t *counts, size_t max_tiles) {
   const uint32_t T = meta[0];
@@ -521,8 +684,8 @@ cudaError_t launch_bucket_t(const Assets &A, const ntc_query *q, size_t n, const
   *launches += 3;
   uint32_t *div_sum = s.meta + meta_words(D) + (D + 1) + 1;
   DecT *dec = reinterpret_cast<DecT *>(s.dec);
-  k_count<DecT><<<chunks, kBucketThreads, smem_count, st>>>(A, q, n, chunks, s.counts, div_sum, dec);
-  e = cudaGetLastError();
+  e = launch_pdl(k_count<DecT>, dim3(chunks), dim3(kBucketThreads), smem_count, st, A, q, n, chunks, s.counts, div_sum,
+                 dec);
   if (e == cudaSuccess)
     e = launch_pdl(k_scan, dim3(D + 1), dim3(1024), 0, st, (const uint32_t *)s.counts, s.offs, chunks, D, s.meta,
                    copy);
@@ -541,11 +704,77 @@ cudaError_t launch_bucket_t(const Assets &A, const ntc_query *q, size_t n, const
 }
 }  // namespace
 
+namespace {
+// Whether one cluster does the whole call: it must fit its CTAs' shared
+// memory.  *items: queries per thread.
+bool small_shape(uint32_t D, size_t n, uint32_t *ctas, uint32_t *items, size_t *smem) {
+  if (n > kSmallMax) return false;
+  // clusters of 16 CTAs where the device schedules them, else of 8
+  static PerDevice attr, most;
+  if (attr.once([]() {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_bucket_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+        if (e != cudaSuccess) return e;
+        return cudaFuncSetAttribute(k_bucket_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      }) != cudaSuccess)
+    return false;
+  const uint32_t most_ctas = (uint32_t)most.value([]() {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kSmallCtas);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = kSmallSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kSmallCtas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_bucket_small, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      clusters = 0;
+    }
+    return clusters > 0 ? (int)kSmallCtas : 8;
+  });
+  uint32_t c = 1;  // CTAs: one query a thread if they suffice
+  while (c < most_ctas && (size_t)c * kSmallThreads < n) c *= 2;
+  if (n > (size_t)c * kSmallThreads * kSmallItems) return false;
+  *ctas = c;
+  *items = (uint32_t)((n + (size_t)c * kSmallThreads - 1) / ((size_t)c * kSmallThreads));
+  *smem = small_smem_bytes(D, *items);
+  return *smem <= (size_t)kSmallSmem;
+}
+
+cudaError_t launch_small(const Assets &A, const ntc_query *q, size_t n, const Scratch &s, uint32_t ctas, uint32_t items,
+                         size_t smem, cudaStream_t st, int *launches) {
+  *launches += 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_bucket_small, A, q, (uint32_t)n, items, s.meta, s.perm, s.sorted);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+}  // namespace
+
 size_t bucket_dec_bytes(uint32_t D) { return D + 1 <= 256 ? 1 : 2; }
 
 cudaError_t launch_bucket(const Assets &A, const ntc_query *q, size_t n, const Scratch &s, cudaStream_t st,
                           int *launches, int copy) {
   if (!s.dec && !copy) return cudaErrorInvalidValue;  // without the decoder array the records are always staged
+  uint32_t ctas, items;
+  size_t smem;
+  if (s.dec && !copy && small_shape(A.num_decoders, n, &ctas, &items, &smem))
+    return launch_small(A, q, n, s, ctas, items, smem, st, launches);
   if (bucket_dec_bytes(A.num_decoders) == 1) return launch_bucket_t<uint8_t>(A, q, n, s, st, launches, copy);
   return launch_bucket_t<uint16_t>(A, q, n, s, st, launches, copy);
 }

@@ -493,7 +493,19 @@ struct TileWalk {
       return;
     }
     if (t >= next) {  // another decoder (next = 0: the first call)
-      while (d < D && tst[d + 1] <= t) ++d;
+      // usually the next decoder; with many small buckets some further, found
+      // by bisection (steps of one took the 586-decoder frame's roles about 20
+      // shared-memory reads per group of tiles)
+      if (d < D && tst[d + 1] <= t) ++d;
+      if (d < D && tst[d + 1] <= t) {
+        uint32_t lo = d + 1, hi = D + 1;  // tst[lo] <= t < tst[hi]
+        while (hi - lo > 1) {
+          const uint32_t mid = (lo + hi) >> 1;
+          if (tst[mid] <= t) lo = mid;
+          else hi = mid;
+        }
+        d = lo;
+      }
       next = d < D ? tst[d + 1] : 0xFFFFFFFFu;
       end = seg[d + 1];
       base = seg[d] - tst[d] * kTile;
