@@ -20,10 +20,15 @@ __device__ __forceinline__ void count_bad(bool bad, unsigned long long *err) {
 // evaluation would.  With one query per thread and the weights broadcast, each
 // 16-byte shared-memory read fed four FMAs and the reads were the bound (31
 // TFLOP/s on a 1080p frame, H = 64); here four of them feed 64.
-// Shared memory: W1^T [16][H], b1, W2^T [H][H], b2, W3^T [H][CP], b3[CP], the
-// activations [H][kActPitch] (feature columns first), the rows' output rows.
-// Tiles are split into contiguous ranges per CTA so a CTA rarely changes
-// decoder.
+// The output layer needs no pass of its own over the activations: a thread
+// multiplies the 8 x 8 second-layer values that it holds by its outputs'
+// columns of W3, and the partial sums of the threads of one query are added
+// from shared memory (read per query and k instead, the output layer took
+// 2,300 shared-memory cycles a tile, a fifth of all).
+// Shared memory: W1^T [16][H], b1, W2^T [H][H], b2, W3 [CP][H], b3[CP], the
+// activations [H][kActPitch] (feature columns first; at the end the partial
+// sums), the rows' output rows.  Tiles are split into contiguous ranges per CTA
+// so a CTA rarely changes decoder.
 constexpr int kActPitch = 132;  // 128 queries and a pad: 16-byte rows, stores of neighbouring rows on other banks
 
 template <int H>
@@ -38,6 +43,11 @@ __device__ __forceinline__ unsigned long long dup2(float x) {
 }
 __device__ __forceinline__ void fma2(unsigned long long &acc, unsigned long long a, unsigned long long b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
 }
 __device__ __forceinline__ float2 unpack2(unsigned long long v) {
   float2 r;
@@ -101,7 +111,7 @@ __global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_f
                                                                                    unsigned long long *err) {
   extern __shared__ float4 smem4[];
   float *sw = reinterpret_cast<float *>(smem4);
-  const float *W1 = sw, *b1 = W1 + H * 16, *W2 = b1 + H, *b2 = W2 + H * H, *W3t = b2 + H, *b3 = W3t + H * CP;
+  const float *W1 = sw, *b1 = W1 + H * 16, *W2 = b1 + H, *b2 = W2 + H * H, *W3 = b2 + H, *b3 = W3 + H * CP;
   const uint32_t D = A.num_decoders, C = W.out_dim;
   float *act = sw + fp32_img_floats(H, C);
   uint32_t *rows = reinterpret_cast<uint32_t *>(act + H * kActPitch);
@@ -151,34 +161,49 @@ __global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_f
     fp32_store<H>(acc, act, q0, o0);
     __syncthreads();
     fp32_layer<H, H>(W2, b2, act, q0, o0, acc);
-    __syncthreads();
-    fp32_store<H>(acc, act, q0, o0);
-    __syncthreads();
-    // the output layer: a thread one query and CP outputs (H = 128: half of them)
-    constexpr int kO = CP * kTile / fp32_threads<H>();
-    const int c0 = (threadIdx.x / kTile) * kO;
-    float o[kO];
 #pragma unroll
-    for (int c = 0; c < kO; ++c) o[c] = b3[c0 + c];
-#pragma unroll 4
-    for (int k = 0; k < H; ++k) {
-      const float h = act[k * kActPitch + r];
-      const float4 *w3 = reinterpret_cast<const float4 *>(W3t + k * CP + c0);
+    for (int o = 0; o < 8; ++o)
 #pragma unroll
-      for (int i = 0; i < kO / 4; ++i) {
-        const float4 x = w3[i];
-        o[4 * i] = fmaf(x.x, h, o[4 * i]);
-        o[4 * i + 1] = fmaf(x.y, h, o[4 * i + 1]);
-        o[4 * i + 2] = fmaf(x.z, h, o[4 * i + 2]);
-        o[4 * i + 3] = fmaf(x.w, h, o[4 * i + 3]);
+      for (int p = 0; p < 4; ++p) {
+        const float2 x = unpack2(acc[p][o]);
+        acc[p][o] = pack2(fmaxf(x.x, 0.0f), fmaxf(x.y, 0.0f));
       }
-    }
     const uint32_t oi = rows[r];
-    if (oi != kNone) {
-      float *o_row = out + (size_t)oi * C;
+    constexpr int kParts = H / 8, kO = 8 * kTile / fp32_threads<H>();  // partial sums of a query; outputs a thread adds up
+    const int part = o0 / 4, c0 = (threadIdx.x / kTile) * kO;
 #pragma unroll
-      for (int c = 0; c < kO; ++c)
-        if (c0 + c < (int)C) o_row[c0 + c] = 1.0f / (1.0f + expf(-o[c]));
+    for (int cb = 0; cb < CP; cb += 8) {  // eight output channels at a time
+      __syncthreads();  // the activations, or the previous channels' sums, have been read
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const float4 w0 = *reinterpret_cast<const float4 *>(W3 + (cb + c) * H + o0);
+        const float4 w1 = *reinterpret_cast<const float4 *>(W3 + (cb + c) * H + o0 + H / 2);
+        const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+        unsigned long long y[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+          const unsigned long long ww = dup2(w[o]);
+#pragma unroll
+          for (int p = 0; p < 4; ++p) fma2(y[p], ww, acc[p][o]);
+        }
+        float *to = act + (part * 8 + c) * kActPitch + q0;
+        *reinterpret_cast<ulonglong2 *>(to) = make_ulonglong2(y[0], y[1]);
+        *reinterpret_cast<ulonglong2 *>(to + 64) = make_ulonglong2(y[2], y[3]);
+      }
+      __syncthreads();
+      float o[kO];
+#pragma unroll
+      for (int c = 0; c < kO; ++c) o[c] = b3[cb + c0 + c];
+#pragma unroll
+      for (int s = 0; s < kParts; ++s)
+#pragma unroll
+        for (int c = 0; c < kO; ++c) o[c] += act[(s * 8 + c0 + c) * kActPitch + r];
+      if (oi != kNone) {
+        float *o_row = out + (size_t)oi * C;
+#pragma unroll
+        for (int c = 0; c < kO; ++c)
+          if (cb + c0 + c < (int)C) o_row[cb + c0 + c] = 1.0f / (1.0f + expf(-o[c]));
+      }
     }
   }
 }
@@ -285,18 +310,15 @@ __global__ void k_pack(const float *w32, uint32_t H, uint32_t C, uint8_t *mma, s
   // fp32 image
   const uint32_t CP = out_pad(C);
   float *f = f32 + (size_t)d * f32_stride;
-  float *fW1 = f, *fb1 = fW1 + H * 16, *fW2 = fb1 + H, *fb2 = fW2 + (size_t)H * H, *fW3t = fb2 + H,
-        *fb3 = fW3t + (size_t)H * CP;
+  float *fW1 = f, *fb1 = fW1 + H * 16, *fW2 = fb1 + H, *fb2 = fW2 + (size_t)H * H, *fW3 = fb2 + H,
+        *fb3 = fW3 + (size_t)H * CP;
   for (uint32_t i = threadIdx.x; i < H * 16; i += blockDim.x) fW1[i] = W1[(i % H) * 16 + i / H];
   for (uint32_t i = threadIdx.x; i < H; i += blockDim.x) {
     fb1[i] = b1[i];
     fb2[i] = b2[i];
   }
   for (uint32_t i = threadIdx.x; i < H * H; i += blockDim.x) fW2[i] = W2[(size_t)(i % H) * H + i / H];
-  for (uint32_t i = threadIdx.x; i < H * CP; i += blockDim.x) {
-    uint32_t j = i / CP, c = i % CP;
-    fW3t[i] = c < C ? W3[(size_t)c * H + j] : 0.0f;
-  }
+  for (uint32_t i = threadIdx.x; i < H * CP; i += blockDim.x) fW3[i] = i / H < C ? W3[i] : 0.0f;
   for (uint32_t i = threadIdx.x; i < CP; i += blockDim.x) fb3[i] = i < C ? b3[i] : 0.0f;
 }
 

@@ -48,8 +48,8 @@ struct Assets {
 //  mma image (fp16/bf16 bits, rows padded by 8 elements so ldmatrix is
 //  conflict-free): W1[H][16+8], W2[H][H+8], W3[16][H+8] (rows >= C zero), then
 //  fp32 biases b1[H], b2[H], b3[16].
-//  fp32 image, transposed: W1^T[16][H], b1[H], W2^T[H][H], b2[H], W3^T[H][CP],
-//  b3[CP] (columns >= C zero), CP = 8 or 16.
+//  fp32 image: W1^T[16][H], b1[H], W2^T[H][H], b2[H], W3[CP][H], b3[CP] (rows
+//  >= C zero), CP = 8 or 16.
 struct WeightImages {
   const uint8_t *mma;       // [D][mma_stride] bytes
   size_t mma_stride;
