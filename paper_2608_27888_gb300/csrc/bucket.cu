@@ -469,8 +469,9 @@ __global__ void __launch_bounds__(kBucketThreads, 5) k_place(Assets A, const ntc
 // further barrier.  Same permutation, tile table and copy decision as the three
 // kernels above, which cost about 16 us of chained launches whatever the size.
 // A whole decode call, with them and this way: 1,000 queries of 16 decoders
-// 20.5 -> 11.2 us, 32,000 20.6 -> 15.5, 65,536 22.6 -> 19.6 (and, by issue on so
-// few SMs, 131,072 24.7 -> 37 with 8 CTAs: hence the limit).
+// 20.5 -> 11.1 us, 32,000 20.6 -> 15.2, 65,536 22.6 -> 18.8. Beyond that the
+// few SMs' issue slots are the bound: 131,072 queries take 27.0 us this way and
+// 22.4 the other.
 constexpr uint32_t kSmallThreads = 1024, kSmallWarps = 32, kSmallCtas = 16, kSmallItems = 4;
 constexpr size_t kSmallMax = (size_t)kSmallCtas * kSmallThreads * kSmallItems;
 
@@ -500,22 +501,23 @@ __device__ __forceinline__ uint32_t cluster_read(const uint32_t *p, uint32_t ran
 
 constexpr int kSmallSmem = 200 * 1024;  // dynamic shared memory of a CTA, at most
 inline size_t small_smem_bytes(uint32_t D, uint32_t items) {
-  return ((size_t)kSmallWarps + 4) * (D + 2) * 4 + (size_t)kSmallThreads * items * 2;
+  return ((size_t)kSmallWarps * (D + 3) + (size_t)4 * (D + 2) + (size_t)kSmallThreads * items) * 4;
 }
 
 __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const ntc_query *q, uint32_t n, uint32_t items,
                                                                 uint32_t *meta, uint32_t *perm, ntc_query *sorted) {
-  // shared memory: per-warp counters [32][D+2]; per decoder the CTA's total,
-  // its place of the CTA's first query, and the scans [D+2] each; the decoders
-  // of the CTA's queries [1024 x items]
+  // shared memory: per-warp counters [32][CW]; per decoder the CTA's total,
+  // its place of the CTA's first query, and the scans [D+2] each; of each of the
+  // CTA's queries its decoder and, from bit 16, its rank among the equal ones of
+  // its warp's run [1024 x items]
   extern __shared__ uint32_t small_sm[];
   __shared__ uint32_t ws[32];
   __shared__ uint32_t s_div;
-  const uint32_t D = A.num_decoders, DW = D + 2;
-  uint32_t *cnt = small_sm, *tot = cnt + kSmallWarps * DW, *gbase = tot + DW, *seg = gbase + DW, *tst = seg + DW;
-  uint16_t *keys = reinterpret_cast<uint16_t *>(tst + DW);
+  const uint32_t D = A.num_decoders, DW = D + 2, CW = DW | 1u;  // (odd: the scan reads columns)
+  uint32_t *cnt = small_sm, *tot = cnt + kSmallWarps * CW, *gbase = tot + DW, *seg = gbase + DW, *tst = seg + DW;
+  uint32_t *keys = tst + DW;
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = cluster_rank(), ctas = cluster_size();
-  for (uint32_t i = threadIdx.x; i < kSmallWarps * DW; i += kSmallThreads) cnt[i] = 0;
+  for (uint32_t i = threadIdx.x; i < kSmallWarps * CW; i += kSmallThreads) cnt[i] = 0;
   if (threadIdx.x == 0) s_div = 0;
   const MapLookup lookup(A);
   const int nbits = key_bits(D);
@@ -525,7 +527,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const 
   const uint32_t run = warp * items * 32;                         // this warp's run in the CTA's queries
   const uint32_t first = rank * items * kSmallThreads + run;      // and in the call's
   const uint32_t *sid = reinterpret_cast<const uint32_t *>(q);
-  uint32_t *my = cnt + warp * DW;
+  uint32_t *my = cnt + warp * CW;
+  const uint32_t lt = (1u << lane) - 1u;
   uint32_t div = 0;
   for (uint32_t it = 0; it < items && first + it * 32 < n; it += 8) {
     uint32_t s[8];
@@ -541,31 +544,30 @@ __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const 
 #pragma unroll
       for (uint32_t v = 1; v < 8; ++v) d = u == v ? s[v] : d;
       if (first + (it + u) * 32 + lane >= n) d = D + 1;  // no query
-      keys[run + (it + u) * 32 + lane] = (uint16_t)d;
       const uint32_t m = match_key(d, nbits);
       const bool leader = lane == (uint32_t)__ffs(m) - 1;
+      keys[run + (it + u) * 32 + lane] = d | (my[d] + __popc(m & lt)) << 16;
+      __syncwarp();
       if (leader) my[d] += __popc(m);
       const uint32_t runs = __popc(__ballot_sync(0xFFFFFFFFu, leader && d <= D));
       div += runs ? runs - 1 : 0u;
       __syncwarp();
     }
   }
-  // runs past the end: no queries
-  for (uint32_t it = 0; it < items; ++it)
-    if (first + it * 32 >= n) keys[run + it * 32 + lane] = (uint16_t)(D + 1);
   if (lane == 0 && div) atomicAdd(&s_div, div);
   __syncthreads();
   for (uint32_t d = warp; d <= D; d += kSmallWarps) {  // the warps' counts of decoder d -> offsets
-    const uint32_t x = cnt[lane * DW + d];
+    const uint32_t x = cnt[lane * CW + d];
     uint32_t y = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t z = __shfl_up_sync(0xFFFFFFFFu, y, o);
       if (lane >= (uint32_t)o) y += z;
     }
-    cnt[lane * DW + d] = y - x;
+    cnt[lane * CW + d] = y - x;
     if (lane == 31) tot[d] = y;
   }
+  __syncwarp();
   cluster_arrive();
   cluster_wait();
   uint32_t all_div = 0;
@@ -581,6 +583,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const 
     tst[d] = (total + kTile - 1) / kTile;
   }
   for (uint32_t r = 0; r < ctas; ++r) all_div += cluster_read(&s_div, r);
+  __syncwarp();
   cluster_arrive();  // (waited for before leaving: no CTA's shared memory goes while others read it)
   __syncthreads();
   block_scan_to(seg, seg, D + 1, ws);
@@ -601,21 +604,20 @@ __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const 
       meta[meta_divergence(D)] = all_div;
     }
   }
-  const uint32_t lt = (1u << lane) - 1u;
-  for (uint32_t it = 0; it < items && first + it * 32 < n; ++it) {
-    const uint32_t d = keys[run + it * 32 + lane], j = first + it * 32 + lane;
-    const uint32_t m = match_key(d, nbits);
-    const uint32_t at = my[d] + __popc(m & lt);
-    __syncwarp();
-    if (lane == (uint32_t)__ffs(m) - 1) my[d] += __popc(m);
-    __syncwarp();
-    if (d > D) continue;
-    const uint32_t p = seg[d] + gbase[d] + at;
+  for (uint32_t d = threadIdx.x; d <= D; d += kSmallThreads) gbase[d] += seg[d];
+  __syncthreads();
+#pragma unroll 4
+  for (uint32_t it = 0; it < items; ++it) {
+    const uint32_t j = first + it * 32 + lane;
+    if (j >= n) break;
+    const uint32_t w = keys[run + it * 32 + lane], d = w & 0xFFFFu;
+    const uint32_t p = gbase[d] + my[d] + (w >> 16);  // (my: the queries of the CTA's earlier warps)
     if (p < n) {
       perm[p] = j;
       if (copy) reinterpret_cast<uint4 *>(sorted)[p] = __ldg(reinterpret_cast<const uint4 *>(q + j));
     }
   }
+  __syncwarp();
   cluster_wait();
 }
 

@@ -45,7 +45,7 @@ def stream(n, S, runs, seed):
 
 
 @pytest.mark.parametrize("runs", [False, True])
-@pytest.mark.parametrize("n", [1, 32, 33, 1024, 1025, 4096, 4097, 8193, 16384, 16385, 32768, 32769, 40001, 65536, 65537])
+@pytest.mark.parametrize("n", [1, 32, 33, 1024, 1025, 4096, 4097, 8193, 16384, 16385, 32768, 32769, 40001, 65536, 65537, 131072, 131073])
 def test_sizes(n, runs):
     S, D = 40, 23
     check(D, S, stream(n, S, runs, n), W.map_random_partition(5, S, D))
