@@ -210,10 +210,10 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
 
 // An activated fp16/bf16 pair of accumulator values.  act 2 evaluates
 // max(h, slope * h) on the packed pair.
-template <bool BF16>
-__device__ __forceinline__ uint32_t pack_act(uint32_t lo, uint32_t hi, uint32_t act, float slope, uint32_t slope2) {
-  if (act == 0) return pack_relu<BF16>(lo, hi);
-  if (act == 2) {
+template <bool BF16, int ACT>
+__device__ __forceinline__ uint32_t pack_act(uint32_t lo, uint32_t hi, float slope, uint32_t slope2) {
+  if (ACT == 0) return pack_relu<BF16>(lo, hi);
+  if (ACT == 2) {
     const uint32_t h = pack<BF16>(__uint_as_float(lo), __uint_as_float(hi));
     uint32_t r;
     if (BF16)
@@ -602,13 +602,14 @@ struct Pipe {
   }
 
   // TMEM accumulator -> activation -> fp16/bf16 pairs -> hidden operand
+  template <int ACT>
   __device__ __forceinline__ void convert(uint32_t ta, uint32_t th) const {
     if constexpr (H == 16) {
       uint32_t v[16], p[8];
       tmem_ld16(ta, v);
       tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 8; ++i) p[i] = pack_act<BF16>(v[2 * i], v[2 * i + 1], act(), P.slope, P.slope2);
+      for (int i = 0; i < 8; ++i) p[i] = pack_act<BF16, ACT>(v[2 * i], v[2 * i + 1], P.slope, P.slope2);
       tmem_st8(th, p);
     } else {
 #pragma unroll
@@ -617,14 +618,20 @@ struct Pipe {
         tmem_ld32(ta + c, v);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 16; ++i) p[i] = pack_act<BF16>(v[2 * i], v[2 * i + 1], act(), P.slope, P.slope2);
+        for (int i = 0; i < 16; ++i) p[i] = pack_act<BF16, ACT>(v[2 * i], v[2 * i + 1], P.slope, P.slope2);
         tmem_st16(th + c / 2, p);
       }
     }
     tmem_wait_st();
   }
 
-  __device__ __forceinline__ void converter(uint32_t e) const {
+  __device__ __forceinline__ void converter(uint32_t e) const {  // (a test per value costs as much as the conversion)
+    if (K1C || P.act == 0) convert_tiles<0>(e);  // the standard shape has ReLU
+    else if (P.act == 2) convert_tiles<2>(e);
+    else convert_tiles<1>(e);
+  }
+  template <int ACT>
+  __device__ __forceinline__ void convert_tiles(uint32_t e) const {
     const uint32_t own = Kg > e ? (Kg - e + NE - 1) / NE : 0, NL = nl();
     uint32_t j = 0;  // the slots' uses
     for (uint32_t g = 0; g < own && !wait.stopped(); g += D, ++j) {
@@ -636,7 +643,7 @@ struct Pipe {
           const uint32_t s = e + NE * s_;
           wait(acc_bar(s), parity);
           fence_after();
-          convert(t_acc(s) + lanes(), t_hid(s) + lanes());
+          convert<ACT>(t_acc(s) + lanes(), t_hid(s) + lanes());
           fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(hid_bar(s));
@@ -644,8 +651,6 @@ struct Pipe {
       }
     }
   }
-  __device__ __forceinline__ uint32_t act() const { return K1C ? 0u : P.act; }  // the standard shape has ReLU
-
   __device__ __forceinline__ void writer(void *out) const {
     const uint32_t row = threadIdx.x & 127, C = P.out_dim;
     float *rowbuf = reinterpret_cast<float *>(smem + P.sm.rows) + (warp & 3) * 32 * PipeSmem::row_words(C);
