@@ -14,9 +14,13 @@
 using namespace ntc;
 
 // ntc_decode_host splits a batch into at most kHostChunks pipelined chunks of
-// at least kHostChunkMin queries.
+// at least kHostChunkMin queries, or kHostChunkMore where that leaves four or
+// more: a chunk's decode has its own bucketing and last wave, and on a 2160p
+// frame (fp16 rows) 2^18-query chunks kept the GPU busier than the host link:
+// 1,165 us with them, 1,074 with 3 * 2^17 and 1,083 with 2^20; a 1080p frame
+// 367, 336 and 390.
 constexpr int kHostChunks = 32;
-constexpr size_t kHostChunkMin = 1u << 18;
+constexpr size_t kHostChunkMin = 1u << 18, kHostChunkMore = 3u << 17;
 
 struct ntc_ctx {
   int device = 0;
@@ -600,7 +604,8 @@ ntc_status ntc_decode_host(ntc_ctx *c, const ntc_query *hq, size_t n, void *vhou
   // same as in one call over all n.  One event per direction serves every
   // chunk: a stream wait takes the event's latest record when it is enqueued.
   size_t chunk = (n + kHostChunks - 1) / kHostChunks;
-  if (chunk < kHostChunkMin) chunk = kHostChunkMin;
+  const size_t least = n / 4 < kHostChunkMin ? kHostChunkMin : n / 4 < kHostChunkMore ? n / 4 : kHostChunkMore;
+  if (chunk < least) chunk = least;
   chunk = (chunk + kBucketChunk - 1) / kBucketChunk * kBucketChunk;
   const size_t nchunks = (n + chunk - 1) / chunk;
   const size_t row = (size_t)c->C * (c->out_half ? 2 : 4);  // bytes of one output row
