@@ -97,6 +97,9 @@ __global__ void __launch_bounds__(kBucketThreads) k_count(Assets A, const ntc_qu
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (uint32_t i = threadIdx.x; i < kWarps * DW; i += blockDim.x) cnt[i] = 0;
   __syncthreads();
+  // a context's map was uploaded when it was created; the allocation-free
+  // entry's (no decoder array) is a copy on the stream just before
+  if (!dec_out) pdl_wait();
   const MapLookup lookup(A);
   const int nbits = key_bits(D);
   const size_t wbase = (size_t)blockIdx.x * kBucketChunk + (size_t)warp * (kBucketItems * 32);
