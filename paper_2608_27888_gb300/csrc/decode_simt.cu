@@ -23,8 +23,7 @@ __device__ __forceinline__ void count_bad(bool bad, unsigned long long *err) {
 // The output layer needs no pass of its own over the activations: a thread
 // multiplies the 8 x 8 second-layer values that it holds by its outputs'
 // columns of W3, and the partial sums of the threads of one query are added
-// from shared memory (read per query and k instead, the output layer took
-// 2,300 shared-memory cycles a tile, a fifth of all).
+// from shared memory (decode 555 -> 534 us).
 // Shared memory: W1^T [16][H], b1, W2^T [H][H], b2, W3 [CP][H], b3[CP], the
 // activations [H][kActPitch] (feature columns first; at the end the partial
 // sums), the rows' output rows.  Tiles are split into contiguous ranges per CTA

@@ -249,15 +249,16 @@ __device__ __forceinline__ void produce_tm(const TmPipe<H, BF16> &pipe, const As
     __half2 acc[kLevels][4];
     accum_taps<true>(taps, acc);
     if (TRI && __any_sync(0xFFFFFFFFu, good && mp.t > 0.0f)) {  // some row blends two mips
+      uint4 raw[kLevels][4];  // both levels' loads in flight
+      float w[kLevels][4];
+      TapIdx th[kLevels];
+#pragma unroll
+      for (int lv = 0; lv < kLevels; ++lv) issue_level_hi<WRAP, DBG>(A, grids, q, good, mp, lv, raw[lv], w[lv], th + lv);
 #pragma unroll
       for (int lv = 0; lv < kLevels; ++lv) {
-        uint4 raw[4];
-        float w[4];
-        TapIdx th;
-        issue_level_hi<WRAP, DBG>(A, grids, q, good, mp, lv, raw, w, &th);
-        if (DBG && good && mp.t > 0.0f) record(lv, 1, raw, w, th);
+        if (DBG && good && mp.t > 0.0f) record(lv, 1, raw[lv], w[lv], th[lv]);
 #pragma unroll
-        for (int t = 0; t < 4; ++t) accum_tap_x2<false>(acc[lv], raw[t], w[t]);
+        for (int t = 0; t < 4; ++t) accum_tap_x2<false>(acc[lv], raw[lv][t], w[lv][t]);
       }
     }
     uint32_t a[8];
