@@ -163,8 +163,8 @@ def peaks():
 
 # the sources each recorded decode kernel is built from
 KERNEL_SOURCES = {
-    "k_decode_tm": ("decode_tc.cuh", "decode_tc.cu", "tcgen05.cuh", "ntc_internal.cuh"),
-    "k_decode_gen_tc": ("decode_gen.cu", "tcgen05.cuh", "ntc_internal.cuh"),
+    "k_decode_tm": ("decode_tc.cuh", "decode_tc.cu", "decode_pipe.cuh", "tcgen05.cuh", "ntc_internal.cuh"),
+    "k_decode_gen_tc": ("decode_gen.cu", "decode_pipe.cuh", "tcgen05.cuh", "ntc_internal.cuh"),
 }
 
 
