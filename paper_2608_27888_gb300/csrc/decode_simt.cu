@@ -26,7 +26,7 @@ __device__ __forceinline__ void count_bad(bool bad, unsigned long long *err) {
 // from shared memory (decode 555 -> 534 us).
 // Shared memory: W1^T [16][H], b1, W2^T [H][H], b2, W3 [CP][H], b3[CP], the
 // activations [H][kActPitch] (feature columns first; at the end the partial
-// sums), the rows' output rows.  Tiles are split into contiguous ranges per CTA
+// sums; the rows' output rows in their pad).  Tiles are split into contiguous ranges per CTA
 // so a CTA rarely changes decoder.
 constexpr int kActPitch = 132;  // 128 queries and a pad: 16-byte rows, stores of neighbouring rows on other banks
 
@@ -101,7 +101,7 @@ __device__ __forceinline__ void fp32_store(const unsigned long long (&acc)[4][8]
 
 inline __host__ __device__ size_t fp32_img_floats(uint32_t H, uint32_t C) { return (f32_image_floats(H, C) + 3) / 4 * 4; }
 inline __host__ __device__ size_t fp32_smem_bytes(uint32_t H, uint32_t C) {
-  return (fp32_img_floats(H, C) + (size_t)H * kActPitch + kTile) * 4;
+  return (fp32_img_floats(H, C) + (size_t)H * kActPitch) * 4;
 }
 
 template <int H, int CP>
@@ -113,7 +113,9 @@ __global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_f
   const float *W1 = sw, *b1 = W1 + H * 16, *W2 = b1 + H, *b2 = W2 + H * H, *W3 = b2 + H, *b3 = W3 + H * CP;
   const uint32_t D = A.num_decoders, C = W.out_dim;
   float *act = sw + fp32_img_floats(H, C);
-  uint32_t *rows = reinterpret_cast<uint32_t *>(act + H * kActPitch);
+  // the rows' output rows, in the activations' pad columns: 512 bytes more and
+  // only three CTAs of H = 64 fit an SM
+  auto row_slot = [&](int i) { return reinterpret_cast<uint32_t *>(act + (i >> 2) * kActPitch + kTile + (i & 3)); };
   constexpr uint32_t kNone = 0xFFFFFFFFu;  // never an output row
   const uint32_t T = __ldg(B.meta);
   const bool copied = rows_copied(B, D);
@@ -150,7 +152,7 @@ __global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_f
       if (valid && !bad) query_features(A, q, f);
 #pragma unroll
       for (int k = 0; k < kInDim; ++k) act[k * kActPitch + r] = f[k];
-      rows[r] = valid && !bad ? oi : kNone;
+      *row_slot(r) = valid && !bad ? oi : kNone;
     }
     if (dec >= D) continue;  // every row was bad
     __syncthreads();
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_f
         const float2 x = unpack2(acc[p][o]);
         acc[p][o] = pack2(fmaxf(x.x, 0.0f), fmaxf(x.y, 0.0f));
       }
-    const uint32_t oi = rows[r];
+    const uint32_t oi = *row_slot(r);
     constexpr int kParts = H / 8, kO = 8 * kTile / fp32_threads<H>();  // partial sums of a query; outputs a thread adds up
     const int part = o0 / 4, c0 = (threadIdx.x / kTile) * kO;
 #pragma unroll
