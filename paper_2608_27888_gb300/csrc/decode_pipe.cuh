@@ -125,9 +125,8 @@ struct Waits {
   __device__ __forceinline__ bool stopped() const { return uniform(*stop) != 0; }
 };
 
-__device__ __forceinline__ void put_elem(float *p, float y) { *p = y; }
-__device__ __forceinline__ void put_elem(__half *p, float y) { *p = __float2half_rn(y); }
-// the same under a predicate: no branch, so that neighbouring elements overlap
+// An output element under a predicate: no branch, so that neighbouring elements
+// overlap.
 __device__ __forceinline__ void put_elem_if(bool on, float *p, float y) {
   asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.global.f32 [%0], %1;\n}\n" ::"l"(p), "f"(y),
                "r"((uint32_t)on)

@@ -73,9 +73,6 @@ __device__ __forceinline__ void fence_before() {
 __device__ __forceinline__ void fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
-__device__ __forceinline__ void wg_bar(int wg) {
-  asm volatile("bar.sync %0, 128;\n" ::"r"(wg + 1) : "memory");
-}
 
 // Shared-memory descriptor of a no-swizzle K-major operand of K columns at
 // addr (16-byte aligned): K-adjacent core matrices 128 bytes apart, 8-row groups
