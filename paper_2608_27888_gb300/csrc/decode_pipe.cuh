@@ -199,14 +199,6 @@ struct RowWriter {
   }
 };
 
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-
 // An activated fp16/bf16 pair of accumulator values.  act 2 evaluates
 // max(h, slope * h) on the packed pair.
 template <bool BF16, int ACT>
@@ -322,6 +314,10 @@ struct Pipe {
     wait.status = status;
     for (uint32_t i = threadIdx.x; i < kOidxRing * 128; i += blockDim.x)
       reinterpret_cast<uint32_t *>(smem + P.sm.oidx)[i] = kNoRow;
+    // an issuer whose wait for the dispatcher has run out reads its word all the
+    // same: until one is written it names image 0 and no commits, so that what it
+    // then issues stays inside the images and the barriers
+    for (uint32_t i = threadIdx.x; i < kOidxRing; i += blockDim.x) *info(i) = 0;
     if (ngrids <= kSmemGrids) {
       GridDesc *g = reinterpret_cast<GridDesc *>(smem + P.sm.grids);
       for (uint32_t i = threadIdx.x; i < ngrids; i += blockDim.x) g[i] = grids[i];
@@ -342,13 +338,9 @@ struct Pipe {
         mbar_init(final_bar(i), 1);
       }
       misc[1] = 0;
-      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+      mbar_init_fence();
     }
-    if (warp == 0) {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(saddr(misc)), "r"(512u)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
+    if (warp == 0) tmem_alloc(saddr(misc));
     fence_before();
     __syncthreads();
     fence_after();
@@ -452,7 +444,7 @@ struct Pipe {
     __syncthreads();
     if (warp == 0) {
       fence_after();
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u) : "memory");
+      tmem_dealloc(tmem);
     }
   }
 
