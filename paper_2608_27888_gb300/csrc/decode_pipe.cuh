@@ -320,16 +320,24 @@ struct Pipe {
     for (uint32_t i = threadIdx.x; i < kOidxRing; i += blockDim.x) *info(i) = 0;
     if (ngrids <= kSmemGrids) {
       GridDesc *g = reinterpret_cast<GridDesc *>(smem + P.sm.grids);
-      for (uint32_t i = threadIdx.x; i < ngrids; i += blockDim.x) g[i] = grids[i];
+      for (uint32_t i = blockDim.x - 1 - threadIdx.x; i < ngrids; i += blockDim.x) g[i] = grids[i];
       grids = g;
     }
-    if (threadIdx.x == 0) {
+    // What a call of a few tiles per CTA takes is mostly this set-up, so its parts
+    // run side by side: the barriers by a thread of the second and one of the
+    // third warp, the allocation by the first, the grid table above by the last
+    // (all by the first warp, one after the other, and the divisions below for
+    // both lists: a 65,536-query raster 6.3 us of GPU time, this way 5.9).
+    if (threadIdx.x == 32) {
       for (uint32_t i = 0; i < 8; ++i) {
         mbar_init(full_bar(i), 5);   // one arrival per producer warp, and the dispatcher's
         mbar_init(empty_bar(i), 1);  // layer 1's commit
         mbar_init(wfull_bar(i), 1);
         mbar_init(wempty_bar(i), NE);  // each issuer's commit
       }
+      mbar_init_fence();
+    }
+    if (threadIdx.x == 64) {
       for (uint32_t i = 0; i < 4; ++i) {
         mbar_init(acc_bar(i), 1);
         mbar_init(hid_bar(i), 4);  // one arrival per converter warp
@@ -373,11 +381,11 @@ struct Pipe {
     // H = 128 single tiles are better on long lists where a decoder has four or
     // more per CTA anyway (four trilinear 2160p frames, 8 decoders: 1,540 ->
     // 1,518 us a call; 586 decoders on 1080p: 128 us against 89 with groups)
-    gshift = all >= 64 * grid ? (H == 128 && all / D_ >= 4 * grid ? 0u : 2u) : all >= 24 * grid ? 1u : 0u;
+    gshift = all >= 64 * grid ? (H == 128 && all >= 4 * grid * D_ ? 0u : 2u) : all >= 24 * grid ? 1u : 0u;
     gstep = (grid - 1) << gshift;
     gfirst = blockIdx.x << gshift;
     K = local(all);
-    Kg = local(good);
+    Kg = good == all ? K : local(good);
   }
 
   // The rows of one producer thread, tile by tile (k = p, p + NP, ...): while

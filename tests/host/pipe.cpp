@@ -169,9 +169,15 @@ static int run(const std::string &mode, uint32_t NL, uint32_t grid, uint32_t cta
   memset(host::smem, 0xEE, sizeof host::smem);  // what an earlier kernel left
   host::bars_at = A.sm.bars, host::img_pitch = A.sm.img_pitch, host::images = A.ns, host::img_bytes = A.img_bytes;
   for (auto &i : host::image_of) i = -1;
-  blockIdx.x = cta, gridDim.x = grid, blockDim.x = 1, threadIdx.x = 0;
-  const GridDesc *grids = nullptr;
-  const P first(A, host::smem, B, D, &host::status_word, grids, 0);
+  blockIdx.x = cta, gridDim.x = grid, blockDim.x = P::kThreads;
+  auto constructed = [&](uint32_t thread) {
+    threadIdx.x = thread;
+    const GridDesc *grids = nullptr;
+    return P(A, host::smem, B, D, &host::status_word, grids, 0);
+  };
+  constructed(0);  // (allocates tensor memory)
+  for (uint32_t i = P::kThreads; i-- > 1;) constructed(i);  // every thread's part of the set-up
+  const P first = constructed(0);
   {
     TileWalk w;
     for (uint32_t k = 0; k < first.K; ++k) {
@@ -183,7 +189,7 @@ static int run(const std::string &mode, uint32_t NL, uint32_t grid, uint32_t cta
   }
   auto warp_of = [&](int warp, auto body) {
     return std::thread([&, warp, body] {
-      blockIdx.x = cta, gridDim.x = grid, blockDim.x = 1024, threadIdx.x = (uint32_t)warp * 32;
+      blockIdx.x = cta, gridDim.x = grid, blockDim.x = P::kThreads, threadIdx.x = (uint32_t)warp * 32;
       P p = first;
       p.warp = warp, p.lane = 0;
       body(p);
