@@ -57,19 +57,21 @@ __device__ __forceinline__ float2 unpack2(unsigned long long v) {
 // acc[q pair][output] = b[output] + sum_k Wt[k][output] * act[k][query]; this
 // thread's queries are q0 .. q0 + 3 and q0 + 64 .. + 67, its outputs o0 .. o0 + 3
 // and o0 + H/2 .. + 3, so that a quarter warp's reads are one 128-byte row.
-template <int H, int K>
+// PAIRS = 2: the first four queries only (the others' sums are zero).
+template <int H, int K, int PAIRS>
 __device__ __forceinline__ void fp32_layer(const float *Wt, const float *b, const float *act, int q0, int o0,
                                            unsigned long long (&acc)[4][8]) {
 #pragma unroll
   for (int o = 0; o < 8; ++o) {
     const unsigned long long v = dup2(b[o0 + (o & 3) + (o >> 2) * (H / 2)]);
 #pragma unroll
-    for (int p = 0; p < 4; ++p) acc[p][o] = v;
+    for (int p = 0; p < 4; ++p) acc[p][o] = p < PAIRS ? v : 0ull;
   }
 #pragma unroll 4
   for (int k = 0; k < K; ++k) {
     const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(act + k * kActPitch + q0);
-    const ulonglong2 a1 = *reinterpret_cast<const ulonglong2 *>(act + k * kActPitch + q0 + 64);
+    ulonglong2 a1 = make_ulonglong2(0, 0);
+    if (PAIRS == 4) a1 = *reinterpret_cast<const ulonglong2 *>(act + k * kActPitch + q0 + 64);
     const float4 w0 = *reinterpret_cast<const float4 *>(Wt + k * H + o0);
     const float4 w1 = *reinterpret_cast<const float4 *>(Wt + k * H + o0 + H / 2);
     const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
@@ -78,8 +80,10 @@ __device__ __forceinline__ void fp32_layer(const float *Wt, const float *b, cons
       const unsigned long long ww = dup2(w[o]);
       fma2(acc[0][o], ww, a0.x);
       fma2(acc[1][o], ww, a0.y);
-      fma2(acc[2][o], ww, a1.x);
-      fma2(acc[3][o], ww, a1.y);
+      if (PAIRS == 4) {
+        fma2(acc[2][o], ww, a1.x);
+        fma2(acc[3][o], ww, a1.y);
+      }
     }
   }
 }
@@ -155,13 +159,23 @@ __global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_f
       *row_slot(r) = valid && !bad ? oi : kNone;
     }
     if (dec >= D) continue;  // every row was bad
+    // This warp's queries are w0 .. w0 + 31 and w0 + 64 .. + 95; short tiles do
+    // without the products past their end.  4,095 decoders with 20,000 queries, a
+    // call at H = 64, 9 channels: 234 us with every tile multiplied in full, 172
+    // this way (one query per thread: 207); 16 with 300,000: 121 and 118.
+    const uint32_t w0 = threadIdx.x / 32 % 2 * 32;
+    const bool some = w0 < len, both = w0 + 64 < len;
+    auto layer = [&](auto k, const float *Wt, const float *b, unsigned long long (&acc)[4][8]) {
+      if (both) fp32_layer<H, decltype(k)::value, 4>(Wt, b, act, q0, o0, acc);
+      else if (some) fp32_layer<H, decltype(k)::value, 2>(Wt, b, act, q0, o0, acc);
+    };
     __syncthreads();
     unsigned long long acc[4][8];
-    fp32_layer<H, kInDim>(W1, b1, act, q0, o0, acc);
+    layer(std::integral_constant<int, kInDim>(), W1, b1, acc);
     __syncthreads();
-    fp32_store<H>(acc, act, q0, o0);
+    if (some) fp32_store<H>(acc, act, q0, o0);
     __syncthreads();
-    fp32_layer<H, H>(W2, b2, act, q0, o0, acc);
+    layer(std::integral_constant<int, H>(), W2, b2, acc);
 #pragma unroll
     for (int o = 0; o < 8; ++o)
 #pragma unroll
@@ -177,9 +191,10 @@ __global__ void __launch_bounds__(fp32_threads<H>(), H == 64 ? 4 : 1) k_decode_f
       __syncthreads();  // the activations, or the previous channels' sums, have been read
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        const float4 w0 = *reinterpret_cast<const float4 *>(W3 + (cb + c) * H + o0);
-        const float4 w1 = *reinterpret_cast<const float4 *>(W3 + (cb + c) * H + o0 + H / 2);
-        const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+        if (!some) break;
+        const float4 wa = *reinterpret_cast<const float4 *>(W3 + (cb + c) * H + o0);
+        const float4 wb = *reinterpret_cast<const float4 *>(W3 + (cb + c) * H + o0 + H / 2);
+        const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
         unsigned long long y[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int o = 0; o < 8; ++o) {
