@@ -82,9 +82,10 @@ typedef struct {
 } ntc_query;
 
 /* Arithmetic of the MLP.  TC_*: tensor cores with fp16/bf16 operands and fp32
- * accumulation; FP32: CUDA-core fp32 reference mode.  Bias and sigmoid are
- * fp32 in every mode; the output rows are fp32 unless ntc_desc.output_format
- * asks for fp16 rows. */
+ * accumulation; FP32: CUDA-core fp32 reference mode.  Biases count
+ * to fp32 accuracy in every mode (|b| up to 2.1e9 where the operands are fp16),
+ * and the sigmoid is fp32; the output rows are fp32 unless
+ * ntc_desc.output_format asks for fp16 rows. */
 typedef enum {
   NTC_PREC_TC_FP16 = 0,
   NTC_PREC_TC_BF16 = 1,

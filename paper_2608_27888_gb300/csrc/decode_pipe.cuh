@@ -24,10 +24,11 @@
 // goes round its D slots layer by layer, so while it converts one tile the
 // tensor pipe multiplies the others.
 //
-// Every layer's bias is one more K step of its MMA: A is a shared block with 1
-// in K columns 0..2, and the weight image's extra 16-wide K block holds the
-// fp32 bias split into three fp16/bf16 parts there, so the accumulator gets the
-// bias to fp32 accuracy and the conversions add nothing.
+// Every layer's bias is one more K step of its MMA: A is a shared block with
+// powers of two in its first K columns (bias_scale), and the weight image's extra
+// 16-wide K block holds the fp32 bias split into as many fp16/bf16 parts, each
+// divided by its column's power: the accumulator gets the bias to fp32 accuracy,
+// and the conversions add nothing.
 //
 // Tiles: CTA b owns the groups b, b + grid, ... of G neighbouring tiles (G = 4
 // for long lists), so at any moment the whole GPU works on neighbouring tiles
@@ -47,7 +48,7 @@ constexpr uint32_t kSmemTileTable = 1024;  // staged when D + 2 <= this
 constexpr uint32_t kSmemGrids = 1024;      // staged when S * levels * mips <= this
 constexpr uint32_t kOidxRing = 16;         // tiles whose output rows are kept (see Pipe)
 constexpr uint32_t kNoRow = 0xFFFFFFFFu;   // never an output row: n <= 2^32 - 256
-constexpr uint32_t kBiasParts = 3;         // K columns of a bias block that carry the bias
+constexpr uint32_t kBiasParts = 4;         // K columns of a bias block that carry the bias
 
 // Shared memory of one launch, as byte offsets: as little as it needs, since
 // what is left of the SM's array is the L1 that holds the gathers.
@@ -100,6 +101,21 @@ inline __host__ __device__ size_t pipe_image_bytes(uint32_t k1, uint32_t H, uint
 // stages of K1 / 2, the ones block (8), T output accumulators of 16.
 constexpr __host__ __device__ uint32_t pipe_columns(uint32_t H, uint32_t T, uint32_t k1, uint32_t stages) {
   return (T * (H + H / 2) + stages * (k1 / 2) + 8 + 15) / 16 * 16 + 16 * T;
+}
+
+// What K column j of the shared A block holds, as a power of two.  A bf16 part
+// has fp32's range, and three of them its 24 bits (the fourth is 0).  An fp16 part
+// has 11 bits between 2^-14 and 2^16, and steps of 2^-24 below: with these powers a
+// bias from 2^-15 to 65,519 * 2^15 (2.1e9) splits exactly, a smaller one to within
+// 2^-39; a larger one is infinite.  (Parts that all count once leave up to 2^-25,
+// and from 65,520 on they are infinite.)
+constexpr __host__ __device__ int bias_scale(bool bf16, uint32_t j) {
+  return bf16 ? 0 : j == 0 ? 15 : j == 1 ? 4 : j == 2 ? -7 : -14;
+}
+// The same as a value of the operand type: two K columns, j and j + 1.
+template <bool BF16>
+constexpr __host__ __device__ uint32_t bias_ones(uint32_t j) {
+  return BF16 ? 0x3F80u | 0x3F80u << 16 : (uint32_t)(bias_scale(false, j) + 15) << 10 | (uint32_t)(bias_scale(false, j + 1) + 15) << 26;
 }
 
 namespace {
@@ -353,9 +369,8 @@ struct Pipe {
     __syncthreads();
     fence_after();
     tmem = uniform(*reinterpret_cast<volatile uint32_t *>(misc));
-    if (warp < 4) {  // the bias operand: 1 in K columns 0, 1 and 2
-      const uint32_t one = BF16 ? 0x3F80u : 0x3C00u;
-      const uint32_t z[8] = {one | one << 16, one, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (warp < 4) {  // the bias operand
+      const uint32_t z[8] = {bias_ones<BF16>(0), bias_ones<BF16>(2), 0u, 0u, 0u, 0u, 0u, 0u};
       tmem_st8(t_ones() + lanes(), z);
       tmem_wait_st();
     }
@@ -752,14 +767,16 @@ struct Pipe {
 };
 
 // One element of a packed bias block: part j (0 .. kBiasParts - 1) of the bias
-// split into values of type T that add up to it.
+// split into values of type T that, times their columns' powers of two, add up to
+// it.  An infinite or NaN part stands alone.
 template <typename T>
 __device__ __forceinline__ T bias_part(float b, uint32_t j) {
   for (uint32_t i = 0;; ++i) {
-    const T h = T(b);
+    const int e = bias_scale(!std::is_same<T, __half>::value, i);
+    const T h = T(ldexpf(b, -e));
     if (i == j) return h;
     if (!isfinite((float)h)) return T(0.0f);
-    b -= (float)h;
+    b -= ldexpf((float)h, e);
   }
 }
 

@@ -7,7 +7,10 @@
 // usage: pipe MODE H GENERAL NL GRID CTA SEED BAD TILES_OF_DECODER...
 //   MODE run: all roles; silent-dispatcher, silent-loader, silent-producer: that
 //   role never starts, so that the others' waits run out.
+// usage: pipe bias BITS...: what the bias block of an fp32 bias adds up to, in fp16
+//   and in bf16 (hexadecimal bits in, exact decimal sums out)
 // Prints one line per violation, and "done".
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -229,8 +232,29 @@ static int run(const std::string &mode, uint32_t NL, uint32_t grid, uint32_t cta
   return 0;
 }
 
+template <typename V>
+static double block_sum(float b) {
+  constexpr bool bf16 = std::is_same<V, __nv_bfloat16>::value;
+  double sum = 0;
+  for (uint32_t j = 0; j < kBiasParts; ++j) {
+    const uint32_t one = bias_ones<bf16>(j & ~1u) >> 16 * (j & 1) & 0xFFFF;
+    const float column = bf16 ? (float)__nv_bfloat16(__nv_bfloat16_raw{(unsigned short)one}) : (float)__half(__half_raw{(unsigned short)one});
+    sum += (double)column * (double)(float)bias_part<V>(b, j);
+  }
+  return sum;
+}
+
 int main(int argc, char **argv) {
   const std::string mode = argv[1];
+  if (mode == "bias") {
+    for (int i = 2; i < argc; ++i) {
+      const uint32_t bits = (uint32_t)strtoul(argv[i], nullptr, 16);
+      float b;
+      memcpy(&b, &bits, 4);
+      printf("%.17g %.17g\n", block_sum<__half>(b), block_sum<__nv_bfloat16>(b));
+    }
+    return 0;
+  }
   const int H = atoi(argv[2]), general = atoi(argv[3]);
   const uint32_t NL = (uint32_t)atoi(argv[4]), grid = (uint32_t)atoi(argv[5]), cta = (uint32_t)atoi(argv[6]);
   const unsigned seed = (unsigned)atoi(argv[7]);

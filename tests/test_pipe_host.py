@@ -8,6 +8,7 @@ import re
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -56,3 +57,17 @@ def test_waits_that_run_out_leave_memory_alone(pipe, shape, silent):
     H, general, layers = shape
     out = pipe("silent-" + silent, H, general, layers, 2, 1, 3, 1, *[3] * 12)
     assert out.endswith("status 1\ndone\n"), out
+
+
+def test_bias_blocks_add_up_to_the_fp32_bias(pipe):
+    rng = np.random.default_rng(3)
+    b = (rng.uniform(1, 2, 4000) * 2.0 ** rng.integers(-30, 30, 4000) * rng.choice([-1, 1], 4000)).astype(np.float32)
+    b = np.concatenate([b, np.array([0, 1, -1, 0.1, 65504, 65536, 70000, -2.0 ** 30, 65519.0 * 2 ** 15, 2.0 ** -15, 2.0 ** -40, np.inf,
+                                     -np.inf, np.nan], np.float32)])
+    got = np.array([[float(x) for x in line.split()] for line in pipe("bias", *(f"{x:08x}" for x in b.view(np.uint32))).splitlines()])
+    half, bf16 = got.T
+    exact = np.abs(b) >= 2.0 ** -15
+    assert np.array_equal(half[exact], b[exact].astype(np.float64))
+    small = np.abs(b) < 2.0 ** -15
+    assert np.abs(half[small] - b[small]).max() <= 2.0 ** -39
+    assert np.array_equal(bf16, b.astype(np.float64), equal_nan=True) and np.isnan(half[-1])
