@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kBucketThreads) k_count(Assets A, const ntc_qu
 #pragma unroll
   for (int it = 0; it < kBucketItems; ++it) {  // every load in flight before any is used
     const size_t j = wbase + it * 32 + lane;
-    s[it] = j < n ? __ldg(sid + 4 * j) : 0u;
+    s[it] = j < n ? sid[4 * j] : 0u;
   }
   uint32_t *my = cnt + warp * DW;
   uint32_t div = 0;  // this warp's groups: distinct decoders - 1
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const 
 #pragma unroll
     for (uint32_t u = 0; u < 8; ++u) {  // eight loads in flight
       const uint32_t j = first + (it + u) * 32 + lane;
-      s[u] = it + u < items && j < n ? __ldg(sid + 4 * (size_t)j) : 0u;
+      s[u] = it + u < items && j < n ? sid[4 * (size_t)j] : 0u;
     }
 #pragma unroll
     for (uint32_t u = 0; u < 8; ++u) s[u] = lookup(A, s[u]);  // every lane: the lookup shuffles
@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const 
     const uint32_t p = gbase[d] + my[d] + (w >> 16);  // (my: the queries of the CTA's earlier warps)
     if (p < n) {
       perm[p] = j;
-      if (copy) reinterpret_cast<uint4 *>(sorted)[p] = __ldg(reinterpret_cast<const uint4 *>(q + j));
+      if (copy) reinterpret_cast<uint4 *>(sorted)[p] = reinterpret_cast<const uint4 *>(q)[j];
     }
   }
   __syncwarp();

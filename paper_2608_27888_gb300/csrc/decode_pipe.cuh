@@ -381,8 +381,8 @@ struct Pipe {
     if (!ident_n && D_ + 2 <= kSmemTileTable) {
       uint32_t *s_seg = reinterpret_cast<uint32_t *>(smem + P.sm.tiles), *s_tst = s_seg + (D_ + 2);
       for (uint32_t i = threadIdx.x; i < D_ + 2; i += blockDim.x) {
-        s_seg[i] = __ldg(seg + i);
-        s_tst[i] = __ldg(tst + i);
+        s_seg[i] = seg[i];
+        s_tst[i] = tst[i];
       }
       seg = s_seg;
       tst = s_tst;
@@ -426,7 +426,7 @@ struct Pipe {
       walk.at(q.seg, q.tst, q.D_, q.tile(k), d, st, len);
       if (row >= len) return;
       pos = st + row;
-      oi_ = q.ident_n ? pos : __ldg(B.perm + pos);
+      oi_ = q.ident_n ? pos : B.perm[pos];
     }
     __device__ __forceinline__ void request() {  // the next tile's record
       if (noi != kNoRow)

@@ -148,6 +148,9 @@ constexpr uint32_t kCopyAboveScore = 4;
 // while its predecessor on the stream is still running; pdl_wait() blocks
 // until that predecessor has completed and its writes are visible (a no-op for
 // an ordinary launch).  pdl_trigger() lets the successor start launching.
+// What a predecessor may have written is read with ordinary or L2 loads after the
+// wait, never with __ldg: that promises memory which nothing writes while the
+// kernel runs, and the kernel may have started before the write.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -417,7 +420,7 @@ __device__ __forceinline__ ntc_query load_query(const ntc_query *q) {
 // Whether the query records of this launch's bucketing were copied (read
 // once the bucketing has finished; false without bucketing).
 __device__ __forceinline__ bool rows_copied(const Buckets &B, uint32_t D) {
-  return !B.identity_n && __ldg(B.meta + meta_copied(D)) != 0u;
+  return !B.identity_n && B.meta[meta_copied(D)] != 0u;
 }
 
 // Row `pos` of the bucketed order: its output row (original index) and query.
