@@ -31,7 +31,8 @@
 // contiguous records.  Equal decoders within a warp are found with one ballot
 // per bit of the decoder id.  The permutation is exactly std::stable_sort of
 // the indices by decoder.
-// Calls of up to 65,536 queries take one launch instead (k_bucket_small).
+// Calls of up to 65,536 queries take one launch instead (k_bucket_small), unless
+// their decoders' counters do not fit its shared memory (above about 1,300).
 #include <algorithm>
 
 #include "ntc_internal.cuh"
@@ -533,29 +534,25 @@ __global__ void __launch_bounds__(kSmallThreads) k_bucket_small(Assets A, const 
   uint32_t *my = cnt + warp * CW;
   const uint32_t lt = (1u << lane) - 1u;
   uint32_t div = 0;
-  for (uint32_t it = 0; it < items && first + it * 32 < n; it += 8) {
-    uint32_t s[8];
+  uint32_t s[kSmallItems];
 #pragma unroll
-    for (uint32_t u = 0; u < 8; ++u) {  // eight loads in flight
-      const uint32_t j = first + (it + u) * 32 + lane;
-      s[u] = it + u < items && j < n ? sid[4 * (size_t)j] : 0u;
-    }
+  for (uint32_t it = 0; it < kSmallItems; ++it) {  // every load in flight before any is used
+    const uint32_t j = first + it * 32 + lane;
+    s[it] = it < items && j < n ? sid[4 * (size_t)j] : 0u;
+  }
 #pragma unroll
-    for (uint32_t u = 0; u < 8; ++u) s[u] = lookup(A, s[u]);  // every lane: the lookup shuffles
-    for (uint32_t u = 0; u < 8 && it + u < items; ++u) {
-      uint32_t d = s[0];
-#pragma unroll
-      for (uint32_t v = 1; v < 8; ++v) d = u == v ? s[v] : d;
-      if (first + (it + u) * 32 + lane >= n) d = D + 1;  // no query
-      const uint32_t m = match_key(d, nbits);
-      const bool leader = lane == (uint32_t)__ffs(m) - 1;
-      keys[run + (it + u) * 32 + lane] = d | (my[d] + __popc(m & lt)) << 16;
-      __syncwarp();
-      if (leader) my[d] += __popc(m);
-      const uint32_t runs = __popc(__ballot_sync(0xFFFFFFFFu, leader && d <= D));
-      div += runs ? runs - 1 : 0u;
-      __syncwarp();
-    }
+  for (uint32_t it = 0; it < kSmallItems; ++it) {
+    if (it >= items || first + it * 32 >= n) break;
+    const uint32_t dl = lookup(A, s[it]);  // every lane: the lookup shuffles
+    const uint32_t d = first + it * 32 + lane < n ? dl : D + 1;  // D + 1: no query
+    const uint32_t m = match_key(d, nbits);
+    const bool leader = lane == (uint32_t)__ffs(m) - 1;
+    keys[run + it * 32 + lane] = d | (my[d] + __popc(m & lt)) << 16;
+    __syncwarp();
+    if (leader) my[d] += __popc(m);
+    const uint32_t runs = __popc(__ballot_sync(0xFFFFFFFFu, leader && d <= D));
+    div += runs ? runs - 1 : 0u;
+    __syncwarp();
   }
   if (lane == 0 && div) atomicAdd(&s_div, div);
   __syncthreads();
