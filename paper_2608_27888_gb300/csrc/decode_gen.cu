@@ -257,14 +257,16 @@ cudaError_t launch_gen_tc_t(const Assets &A, const GenWeights &G, const Buckets 
   const uint32_t stages = pipe_columns(H, S::T, G.k1, S::NP) <= 512 ? S::NP : 2;
   static_assert(pipe_columns(H, S::T, kGenMaxIn - 16, 2) <= 512, "tensor memory plan exceeds 512 columns");
   if (pipe_columns(H, S::T, G.k1, stages) > 512) return cudaErrorInvalidConfiguration;
-  // images in shared memory: one per slot or more, so that the next decoder's
-  // weights arrive early (at H = 128 any number works: Pipe)
+  // images in shared memory: four, one per slot or more, so that the next
+  // decoder's weights arrive early; at H = 128, where any number works (Pipe), as
+  // many as fit (four hidden layers: one)
   uint32_t ns = 4;
+  static_assert(H == 128 || S::T <= 4, "an image per slot");
   auto args = [&]() {
     return pipe_args(G.tc, G.tc_stride, G.k1, H, G.layers, ns, S::NP, stages, ngrids, A.num_decoders, G.out_dim, G.out_half, out, n);
   };
   PipeArgs P = args();
-  while (ns > (H == 128 ? 1u : (uint32_t)S::T) && P.sm.total > (H == 128 ? kMostSmem : 131072u)) {
+  while (H == 128 && ns > 1 && P.sm.total > kMostSmem) {
     --ns;
     P = args();
   }

@@ -163,12 +163,10 @@ static int run(const std::string &mode, uint32_t NL, uint32_t grid, uint32_t cta
   Buckets B{};
   B.meta = meta.data();
   const uint32_t stages = pipe_columns(H, T, k1, NP) <= 512 ? NP : 2;
-  PipeArgs A = pipe_args(nullptr, 1, k1, H, NLC ? NLC : NL, 1, NP, stages, 0, D, 9, 0, nullptr, seg);
-  uint32_t ns = 4;  // the launches' rule
-  for (;; --ns) {
-    A = pipe_args(nullptr, 1, k1, H, NLC ? NLC : NL, K1C ? (uint32_t)T : ns, NP, stages, 0, D, 9, 0, nullptr, seg);
-    if (K1C || ns == (H == 128 ? 1u : (uint32_t)T) || A.sm.total <= (H == 128 ? 232448u : 131072u)) break;
-  }
+  uint32_t ns = K1C ? (uint32_t)T : 4;  // the launches' rule
+  auto args = [&] { return pipe_args(nullptr, 1, k1, H, NLC ? NLC : NL, ns, NP, stages, 0, D, 9, 0, nullptr, seg); };
+  PipeArgs A = args();
+  while (!K1C && H == 128 && ns > 1 && A.sm.total > 232448) --ns, A = args();
   memset(host::smem, 0xEE, sizeof host::smem);  // what an earlier kernel left
   host::bars_at = A.sm.bars, host::img_pitch = A.sm.img_pitch, host::images = A.ns, host::img_bytes = A.img_bytes;
   for (auto &i : host::image_of) i = -1;
