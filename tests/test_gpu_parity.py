@@ -552,30 +552,38 @@ def test_a_wait_that_gives_up_is_reported_and_the_context_recovers():
     check_tc(got, ref, "after a wait gave up")
 
 
-@pytest.mark.parametrize("hidden,out_dim,mips", [(64, 8, 1), (128, 9, 2)])
-def test_every_tile_switches_decoder(hidden, out_dim, mips):
-    """The most decoder changes the tensor-core decode can meet: 4095 decoders
-    of exactly 8 tiles (1024 queries) each, so the next tile of every consumer
-    (4 x 152 tiles later at H = 64, 2 x 152 at H = 128) belongs to another
-    decoder and the weight image is reloaded before every tile.  The reload must
-    wait for the previous tile's output layer, which still reads W3 of the
-    image (Sec. 3.3: every row is decoded by its own decoder D_c(i)).  Every row
-    is compared with the oracle."""
-    D, per = 4095, 1024
+DEEP = dict(levels=1, channels=4, pe_frequencies=6, activation=1, layers=4)  # H = 128: one image in shared memory
+
+
+@pytest.mark.parametrize("hidden,out_dim,mips,runs,general,precision", [
+    (64, 8, 1, "eight tiles", {}, "fp16"), (128, 9, 2, "eight tiles", {}, "fp16"),
+    (64, 9, 1, "a tile", {}, "fp16"), (128, 8, 1, "a tile", {}, "bf16"), (128, 9, 1, "a tile", DEEP, "fp16"),
+    (64, 8, 1, "one to three", {}, "bf16"), (128, 9, 1, "one to three", {}, "fp16"),
+    (128, 9, 1, "one to three", DEEP, "bf16"), (64, 9, 1, "one to three", DEEP, "fp16")])
+def test_every_tile_switches_decoder(hidden, out_dim, mips, runs, general, precision):
+    """Many decoder changes: 4095 decoders of one ragged tile each, so that the
+    weights change with every tile of a CTA (27 of them on 152 SMs); of one to three
+    tiles; and of eight, on a list long enough that a CTA takes groups of four
+    neighbouring tiles.  An image is loaded again once the last MMA that reads it
+    has completed, at the latest the output layer's of its decoder's last tile
+    (Sec. 3.3: every row is decoded by its own decoder D_c(i)).  Every row is
+    compared with the oracle."""
+    D = 4095
     seed = W.BASE_SEED + 900 + hidden
-    a = W.make_assets(seed, D, 16, mips, D, W.map_identity(D), hidden=hidden, out_dim=out_dim)
-    n = D * per
+    a = W.make_assets(seed, D, 16, mips, D, W.map_identity(D), hidden=hidden, out_dim=out_dim, **general)
     rng = np.random.default_rng(seed)
+    per = {"eight tiles": np.full(D, 1024), "a tile": rng.integers(1, 129, D), "one to three": rng.integers(1, 385, D)}[runs]
+    n = int(per.sum())
     q = np.zeros(n, dtype=W.QUERY_DTYPE)
     q["set_id"] = rng.permutation(np.repeat(np.arange(D, dtype=np.uint32), per))
     q["u"] = rng.random(n, dtype=np.float32)
     q["v"] = rng.random(n, dtype=np.float32)
     q["lod"] = rng.random(n, dtype=np.float32) if mips > 1 else 0.0
     ref, _ = oracle.decode(a, q)
-    dec = ntc().Decoder(a, "fp16")
+    dec = ntc().Decoder(a, precision)
     for _ in range(2):
         got = dec.decode(dq(q)).cpu().numpy()
-        check_tc(got, ref, f"H={hidden} every tile a new decoder")
+        check_tc(got, ref, f"H={hidden}, {runs} a decoder")
     assert dec.error_count() == 0
     dec.close()
     torch.cuda.empty_cache()
