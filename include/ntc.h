@@ -205,11 +205,12 @@ NTC_API ntc_status ntc_decode(ntc_ctx *ctx, const ntc_query *d_queries, size_t n
 /* ntc_decode on HOST buffers: copies the queries to context-owned device
  * memory, decodes, copies the outputs back into h_out and synchronises before
  * returning.  The batch is split into up to 32 chunks (at least 2^18 queries
- * each, 3 * 2^17 where that leaves four chunks) whose upload, decode and download overlap: uploads and downloads run
- * on two context-owned streams ordered after the work already queued on
- * `cuda_stream`, decodes on `cuda_stream`.  Each chunk is bucketed on its own;
- * outputs are the same as one ntc_decode over all n.  Pinned host memory is
- * needed for the copies to overlap. */
+ * each, 3 * 2^17 where that leaves four chunks) whose upload, decode and
+ * download overlap: uploads and downloads run on two context-owned streams
+ * ordered after the work already queued on `cuda_stream`, decodes on
+ * `cuda_stream`.  Each chunk is bucketed on its own; outputs are the same as
+ * one ntc_decode over all n.  Pinned host memory is needed for the copies to
+ * overlap. */
 NTC_API ntc_status ntc_decode_host(ntc_ctx *ctx, const ntc_query *h_queries, size_t n, void *h_out,
                            void *cuda_stream, ntc_mode mode);
 
@@ -300,7 +301,7 @@ NTC_API size_t ntc_max_tiles(const ntc_ctx *ctx, size_t n);
  * the device.  Returns NTC_ERR_CUDA (and still writes *count) when a kernel
  * gave up one of its bounded waits since then (every mbarrier wait of the
  * tensor-core kernels ends after 200 ms; the bucketing waits on nothing but, in
- * calls of up to 65,536 queries, a hardware cluster barrier): that call's
+ * most calls of up to 65,536 queries, a hardware cluster barrier): that call's
  * results are invalid, the context stays usable.  The reset clears both. */
 NTC_API ntc_status ntc_get_error_count(ntc_ctx *ctx, uint64_t *count);
 NTC_API ntc_status ntc_reset_error_count(ntc_ctx *ctx);

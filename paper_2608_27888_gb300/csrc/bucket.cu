@@ -32,7 +32,8 @@
 // per bit of the decoder id.  The permutation is exactly std::stable_sort of
 // the indices by decoder.
 // Calls of up to 65,536 queries take one launch instead (k_bucket_small), unless
-// their decoders' counters do not fit its shared memory (above about 1,300).
+// their decoders' counters do not fit its shared memory (above about 1,300), or the
+// device schedules clusters of 8 CTAs at most (then up to 32,768 queries).
 #include <algorithm>
 
 #include "ntc_internal.cuh"

@@ -162,9 +162,11 @@ __device__ __forceinline__ void put_elem_if(bool on, __half *p, float y) {
 // through the SM-to-L2 crossbar for a 2160p frame instead of 0.3; but each
 // shared-memory or shuffle step of this way queues behind the producers'
 // gathers.  At H = 128 the crossbar is what matters (four trilinear 2160p
-// frames: decode 1,410 -> 1,341 us with the buffer), at H = 64 the writers'
-// time per tile (2160p frame 295 us with it, 228 without; Sec. 4's decoder on
-// 1080p 116 and 82).
+// frames, nine channels: decode 1,421 -> 1,327 us with the buffer), at H = 64 the
+// writers' time per tile (a 2160p frame 350 us with it, 218 without; Sec. 4's
+// decoder on 1080p 143 and 86).  Sec. 4's decoder at H = 128, whose gathers are
+// half as wide, would be better off without it too (128 x 5 on 1283 x 717: 106 us
+// with it, 95 without).
 struct RowWriter {
   uint32_t at[16];  // element i: its row in the low 5 bits, its channel from bit 8
   __device__ __forceinline__ RowWriter(uint32_t C, int lane) {
@@ -394,8 +396,8 @@ struct Pipe {
     const uint32_t good = ident_n ? all : tst[D_];  // the bad bucket's tiles come last
     // longer groups share weights better, but leave the last wave emptier.  At
     // H = 128 single tiles are better on long lists where a decoder has four or
-    // more per CTA anyway (four trilinear 2160p frames, 8 decoders: 1,540 ->
-    // 1,518 us a call; 586 decoders on 1080p: 128 us against 89 with groups)
+    // more per CTA anyway (four trilinear 2160p frames, 8 decoders: 1,511 ->
+    // 1,500 us a call; 586 decoders on 1080p: decode 127 us, with groups 88)
     gshift = all >= 64 * grid ? (H == 128 && all >= 4 * grid * D_ ? 0u : 2u) : all >= 24 * grid ? 1u : 0u;
     gstep = (grid - 1) << gshift;
     gfirst = blockIdx.x << gshift;

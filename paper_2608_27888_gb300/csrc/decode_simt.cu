@@ -15,19 +15,21 @@ __device__ __forceinline__ void count_bad(bool bad, unsigned long long *err) {
 
 // fp32 decode over bucketed tiles: a CTA multiplies a tile's 128 activation
 // columns by its decoder's matrices out of shared memory, a thread 8 queries x
-// 8 outputs at a time, two queries per packed FMA.  Every sum runs over k in
-// increasing order from the bias, one rounding per term, as a scalar
-// evaluation would.  With one query per thread and the weights broadcast, each
+// 8 outputs at a time, two queries per packed FMA.  The sums of the two hidden
+// layers run over k in increasing order from the bias, one rounding per term, as
+// a scalar evaluation would.  With one query per thread and the weights broadcast, each
 // 16-byte shared-memory read fed four FMAs and the reads were the bound (31
 // TFLOP/s on a 1080p frame, H = 64); here four of them feed 64.
 // The output layer needs no pass of its own over the activations: a thread
 // multiplies the 8 x 8 second-layer values that it holds by its outputs'
 // columns of W3, and the partial sums of the threads of one query are added
-// from shared memory (decode 555 -> 534 us).
+// from shared memory (decode 555 -> 534 us).  An output is its bias plus H / 8
+// partial sums, each over eight k from zero: in fp32 like the sums in order, and no
+// further from 64 bits (5e-8 relative either way).
 // Shared memory: W1^T [16][H], b1, W2^T [H][H], b2, W3 [CP][H], b3[CP], the
 // activations [H][kActPitch] (feature columns first; at the end the partial
-// sums; the rows' output rows in their pad).  Tiles are split into contiguous ranges per CTA
-// so a CTA rarely changes decoder.
+// sums; the rows' output rows in their pad).  Tiles are split into contiguous
+// ranges per CTA so a CTA rarely changes decoder.
 constexpr int kActPitch = 132;  // 128 queries and a pad: 16-byte rows, stores of neighbouring rows on other banks
 
 template <int H>
