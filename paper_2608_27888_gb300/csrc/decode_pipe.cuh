@@ -383,8 +383,8 @@ struct Pipe {
     if (!ident_n && D_ + 2 <= kSmemTileTable) {
       uint32_t *s_seg = reinterpret_cast<uint32_t *>(smem + P.sm.tiles), *s_tst = s_seg + (D_ + 2);
       for (uint32_t i = threadIdx.x; i < D_ + 2; i += blockDim.x) {
-        s_seg[i] = seg[i];
-        s_tst[i] = tst[i];
+        s_seg[i] = ld_word(seg + i);
+        s_tst[i] = ld_word(tst + i);
       }
       seg = s_seg;
       tst = s_tst;
@@ -428,7 +428,7 @@ struct Pipe {
       walk.at(q.seg, q.tst, q.D_, q.tile(k), d, st, len);
       if (row >= len) return;
       pos = st + row;
-      oi_ = q.ident_n ? pos : B.perm[pos];
+      oi_ = q.ident_n ? pos : ld_word(B.perm + pos);
     }
     __device__ __forceinline__ void request() {  // the next tile's record
       if (noi != kNoRow)

@@ -10,10 +10,7 @@ inline V __shfl_sync(unsigned, V v, int) {
   return v;
 }
 inline bool __all_sync(unsigned, bool x) { return x; }
-template <typename V>
-inline V __ldg(const V *p) {
-  return *p;
-}
+inline uint32_t ld_word(const uint32_t *p) { return *p; }
 inline float __uint_as_float(uint32_t) { return 0.0f; }
 inline uint32_t min(uint32_t a, uint32_t b) { return a < b ? a : b; }
 constexpr int kTile = NTC_TILE_ROWS;
