@@ -345,7 +345,8 @@ struct Pipe {
     // run side by side: the barriers by a thread of the second and one of the
     // third warp, the allocation by the first, the grid table above by the last
     // (all by the first warp, one after the other, and the divisions below for
-    // both lists: a 65,536-query raster 6.3 us of GPU time, this way 5.9).
+    // both lists also where they are the same: a 65,536-query raster 6.2 us of GPU
+    // time, this way 5.6).
     if (threadIdx.x == 32) {
       for (uint32_t i = 0; i < 8; ++i) {
         mbar_init(full_bar(i), 5);   // one arrival per producer warp, and the dispatcher's
@@ -398,11 +399,15 @@ struct Pipe {
     // H = 128 single tiles are better on long lists where a decoder has four or
     // more per CTA anyway (four trilinear 2160p frames, 8 decoders: 1,511 ->
     // 1,500 us a call; 586 decoders on 1080p: decode 127 us, with groups 88)
-    gshift = all >= 64 * grid ? (H == 128 && all >= 4 * grid * D_ ? 0u : 2u) : all >= 24 * grid ? 1u : 0u;
+    gshift = all >= 64 * grid ? (H == 128 && all / D_ >= 4 * grid ? 0u : 2u) : all >= 24 * grid ? 1u : 0u;
     gstep = (grid - 1) << gshift;
     gfirst = blockIdx.x << gshift;
-    K = local(all);
-    Kg = good == all ? K : local(good);
+    if (good == all) {
+      K = Kg = local(all);
+    } else {
+      K = local(all);
+      Kg = local(good);
+    }
   }
 
   // The rows of one producer thread, tile by tile (k = p, p + NP, ...): while
