@@ -473,10 +473,11 @@ __global__ void __launch_bounds__(kBucketThreads, 5) k_place(Assets A, const ntc
 // distributed shared memory, and every warp then places its own run with no
 // further barrier.  Same permutation, tile table and copy decision as the three
 // kernels above, which cost about 16 us of chained launches whatever the size.
-// A whole decode call, with them and this way: 1,000 queries of 16 decoders
-// 20.5 -> 11.1 us, 32,000 20.6 -> 15.2, 65,536 22.6 -> 18.8. Beyond that the
-// few SMs' issue slots are the bound: 131,072 queries take 27.0 us this way and
-// 22.4 the other.
+// A whole decode call, with them and this way (GPU time): 1,000 queries of 16
+// decoders 15.1 -> 9.6 us, 32,000 17.3 -> 13.9, 65,536 18.5 -> 17.3; 65,536 of 300
+// 29.0 -> 23.0, of 1,200 47.0 -> 40.9.  Beyond that the few SMs' issue slots are
+// the bound: 131,072 queries of 16 took 27.0 us this way and 22.4 the other (a build
+// with eight queries a thread).
 constexpr uint32_t kSmallThreads = 1024, kSmallWarps = 32, kSmallCtas = 16, kSmallItems = 4;
 constexpr size_t kSmallMax = (size_t)kSmallCtas * kSmallThreads * kSmallItems;
 
